@@ -603,6 +603,7 @@ struct LevelPlan {
     size_t light_smem_bytes = 0;  // light vertices: kLightThreads CTAs, segment-search map
     int light_occupancy = 0;
     int micro_occupancy = 0;      // tiny vertices: the warp-per-vertex kernel
+    int dense_occupancy = 0;      // many pulled entries: direct addressing (0: not used)
 };
 
 struct Builder {
@@ -1020,12 +1021,36 @@ struct Builder {
             }
             for (int b = 0; b < kLightBucket; ++b)
                 (warp_level && b < kMicroBucket ? n_micro : n_light) += hstt->bucket_cnt[b];
-            const int n_heavy = hstt->n_smem - n_light - n_micro;
+            int n_dense = 0;
+            for (int b = kDenseBucket; b < kBuckets; ++b) n_dense += hstt->bucket_cnt[b];
+            const int n_heavy = hstt->n_smem - n_light - n_micro - n_dense;
             A.granular = o.granular ? 1 : 0;
+            size_t slab = 0;
+            int dense_grid = 0;
+            if (n_dense > 0) {
+                // candidate slabs of 12 bytes an entry, one per persistent
+                // CTA; granular builds leave half of every SM
+                A.cap_c_max = ((uint32_t)hstt->need_cap_d + 31) & ~31u;
+                slab = (size_t)A.cap_c_max * 12;
+                dense_grid = std::min(n_dense, sms * (o.granular ? std::max(1, plan.dense_occupancy / 2) : plan.dense_occupancy));
+                dense_grid = (int)std::min<size_t>(dense_grid, std::max<size_t>(1, ((size_t)4 << 30) / slab));
+                if (o.max_ctas > 0) dense_grid = std::min(dense_grid, o.max_ctas);
+                const int rc = ensure_gscratch(slab * dense_grid);
+                if (rc) return rc;
+            }
             cudaEventRecord(ek0, st);
             cudaError_t e = cudaSuccess;
-            if (n_heavy > 0) {
+            if (n_dense > 0) {
                 A.items = items;
+                A.n_items = n_dense;
+                A.work = &stt->work_dense;
+                A.gscratch = gscratch;
+                A.gscratch_stride = slab;
+                e = launch_level_dense(dense_grid, A, st);
+                out.launches += 1;
+            }
+            if (e == cudaSuccess && n_heavy > 0) {
+                A.items = items + n_dense;
                 A.n_items = n_heavy;
                 A.work = &stt->work_smem;
                 A.cap_c_max = plan.cap_c;
@@ -1038,7 +1063,7 @@ struct Builder {
                 out.launches += 1;
             }
             if (e == cudaSuccess && n_light > 0) {
-                A.items = items + n_heavy;
+                A.items = items + n_dense + n_heavy;
                 A.n_items = n_light;
                 A.work = &stt->work_light;
                 A.cap_c_max = kLightCap;
@@ -1051,7 +1076,7 @@ struct Builder {
                 out.launches += 1;
             }
             if (e == cudaSuccess && n_micro > 0) {  // one warp per vertex
-                A.items = items + n_heavy + n_light;
+                A.items = items + n_dense + n_heavy + n_light;
                 A.n_items = n_micro;
                 A.work = &stt->work_micro;
                 const int per_cta = kMicroThreads / 32;
@@ -1151,6 +1176,11 @@ struct Builder {
         if (plan.light_occupancy < 1) return PSPC_E_INVAL;
         PSPC_TRY_CUDA(micro_kernel_occupancy(&plan.micro_occupancy));
         if (plan.micro_occupancy < 1) return PSPC_E_INVAL;
+        // Direct addressing with the automatic tables only: a caller that
+        // asks for smaller ones, a map kind or the push buckets gets the
+        // hash kernels.
+        if (plan.dense_occupancy == 0 && o.map_kind == 0 && o.cand_capacity >= 4096 && o.paradigm == 0)
+            PSPC_TRY_CUDA(dense_kernel_attrs(&plan.dense_occupancy));
         return PSPC_OK;
     }
 
@@ -1278,10 +1308,13 @@ struct Builder {
                 ce = launch_dense_prefix(d, n, seg, hub_arena, comp_base, hpre, st);
                 out.launches += 1;
             }
+            // the largest count of level d-1 (level 1: every count is 1)
+            const DenseRule dense{plan.dense_occupancy > 0, d == 2 ? 1u : hstt->cmax,
+                                  o.granular ? kDenseMinRawGranular : kDenseMinRaw, comp_base};
             if (ce == cudaSuccess)
                 ce = launch_cost(d, n, arcs, rp_r, col_r, arc_src, seg + (int64_t)(d - 1) * n, hub_arena,
                                  skip_prefix ? hpre : nullptr, arc_lo, cnt_arc, raw_u, lab_size, stt,
-                                 plan.label_limit, glist, items, st, &out.launches);
+                                 plan.label_limit, dense, glist, items, st, &out.launches);
             if ((rc = cuda_status(ce))) break;
             if ((rc = read_status())) break;
             if (hstt->n_active == 0) break;
@@ -1326,6 +1359,8 @@ struct Builder {
                 keep.n_retry = 0;
                 keep.arena_overflow = 0;
                 keep.work_smem = keep.work_global = keep.work_light = keep.work_giant = keep.work_micro = 0;
+                keep.work_dense = 0;
+                keep.cmax = 0;
                 keep.n_giant = 0;
                 memset(keep.route_att, 0, sizeof(keep.route_att));  // the level is re-run from scratch
                 memset(keep.route_ovf, 0, sizeof(keep.route_ovf));

@@ -151,9 +151,17 @@ __global__ void __launch_bounds__(kPrefixWarps * 32)
     if (lane == 0) hpre[u] = (int32_t)(H < (uint32_t)u ? H : (uint32_t)u);
 }
 
+// Bucket of a vertex: floor(log2 pulled entries) (at most kDenseBucket - 1),
+// or kDenseBucket more for the dense kernel's vertices, which come first.
+__device__ __forceinline__ int bucket_of(const DenseRule& R, int64_t raw, int64_t span, int64_t deg) {
+    const int b = 63 - __clzll((unsigned long long)raw);
+    if (dense_vertex(R, raw, span, deg)) return kDenseBucket + b;
+    return b < kDenseBucket ? b : kDenseBucket - 1;
+}
+
 __global__ void k_cost_vertices(int64_t n, const int64_t* __restrict__ rp, const uint64_t* __restrict__ seg_prev,
                                 const int64_t* __restrict__ raw_u, int64_t* __restrict__ lab_size, LevelStatus* stt,
-                                int64_t label_limit, int32_t* __restrict__ glist) {
+                                int64_t label_limit, const DenseRule dense, int32_t* __restrict__ glist) {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= n) return;
     const int64_t ls = lab_size[u] + seg_len(seg_prev[u]);
@@ -165,7 +173,10 @@ __global__ void k_cost_vertices(int64_t n, const int64_t* __restrict__ rp, const
     atomicAdd(&stt->n_active, 1);
     if (ls <= label_limit) {
         atomicAdd(&stt->n_smem, 1);
-        atomicAdd(&stt->bucket_cnt[63 - __clzll((unsigned long long)raw)], 1);
+        const int64_t span = u - (dense.comp_base ? dense.comp_base[u] : 0);
+        const int b = bucket_of(dense, raw, span, rp[u + 1] - rp[u]);
+        if (b >= kDenseBucket) atomicMax(&stt->need_cap_d, (unsigned long long)(raw < span ? raw : span));
+        atomicAdd(&stt->bucket_cnt[b], 1);
     } else {
         const int p = atomicAdd(&stt->n_global, 1);
         glist[p] = (int32_t)u;
@@ -184,13 +195,15 @@ __global__ void k_bucket_base(LevelStatus* stt) {
     }
 }
 
-__global__ void k_bucket_fill(int64_t n, const int64_t* __restrict__ raw_u, const int64_t* __restrict__ lab_size,
-                              LevelStatus* stt, int64_t label_limit, int32_t* __restrict__ items) {
+__global__ void k_bucket_fill(int64_t n, const int64_t* __restrict__ rp, const int64_t* __restrict__ raw_u,
+                              const int64_t* __restrict__ lab_size, LevelStatus* stt, int64_t label_limit,
+                              const DenseRule dense, int32_t* __restrict__ items) {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= n) return;
     const int64_t raw = raw_u[u];
     if (raw == 0 || lab_size[u] > label_limit) return;
-    const int b = 63 - __clzll((unsigned long long)raw);
+    const int64_t span = u - (dense.comp_base ? dense.comp_base[u] : 0);
+    const int b = bucket_of(dense, raw, span, rp[u + 1] - rp[u]);
     items[stt->bucket_base[b] + atomicAdd(&stt->bucket_fill[b], 1)] = (int32_t)u;
 }
 
@@ -311,6 +324,12 @@ __device__ __forceinline__ bool cand_insert(uint32_t* keys, unsigned long long* 
     }
     *(volatile int*)abort_flag = 1;
     return false;
+}
+
+// A count as LevelStatus::cmax keeps it: saturated where it or its flag
+// says 2^32 or more.
+__device__ __forceinline__ uint32_t count_bound(uint64_t c, uint32_t ovf) {
+    return (ovf != 0 || (c >> 32) != 0) ? 0xFFFFFFFFu : (uint32_t)c;
 }
 
 __device__ __forceinline__ long long warp_incl_scan64(long long v) {
@@ -699,6 +718,7 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kWarps = NT / 32;
     const uint64_t* seg_prev = A.seg + (int64_t)(d - 1) * n;
+    uint32_t cm = 0;  // largest count appended by this thread (LevelStatus::cmax)
 
     for (int round = 0;; ++round) {
         if (tid == 0) s_item = A.granular ? (round == 0 ? (int)blockIdx.x : A.n_items) : atomicAdd(A.work, 1);
@@ -1072,8 +1092,10 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                         const uint32_t h = key & kHubMask;
                         const uint32_t hr = h - cbase;
                         const uint32_t r = wp[hr >> 5] + __popc(sb[hr >> 5] & ((1u << (hr & 31)) - 1u));
+                        const uint64_t cv = ccnt[slot];
                         A.hub_arena[b0 + r] = h | (key & kOvfBit);
-                        A.cnt_arena[b0 + r] = ccnt[slot];
+                        A.cnt_arena[b0 + r] = cv;
+                        cm = max(cm, count_bound(cv, key & kOvfBit));
                     }
                     if (tid == 0) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
                 }
@@ -1103,8 +1125,10 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                     for (int i = tid; i < S; i += NT) {
                         const uint32_t slot = (uint32_t)sortbuf[i];
                         const uint32_t key = ckeys[slot];
+                        const uint64_t cv = ccnt[slot];
                         A.hub_arena[b0 + i] = (key & kHubMask) | (key & kOvfBit);
-                        A.cnt_arena[b0 + i] = ccnt[slot];
+                        A.cnt_arena[b0 + i] = cv;
+                        cm = max(cm, count_bound(cv, key & kOvfBit));
                     }
                     if (tid == 0) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
                 }
@@ -1114,7 +1138,11 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         if (tid == 0 && may_overflow) atomicAdd(&A.stt->route_att[rb], 1u);
         __syncthreads();
     }
+    cm = __reduce_max_sync(0xFFFFFFFFu, cm);
+    if (lane == 0 && cm) atomicMax(&A.stt->cmax, cm);
 }
+
+#include "pspc_dense.cuh"
 
 // ---------------------------------------------------------------------------
 // The level for tiny vertices (fewer than 2^kMicroBucket pulled entries):
@@ -1150,6 +1178,7 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
     uint32_t* ul = s_lmkw[w];
     const unsigned lt = (1u << lane) - 1u;
     unsigned long long n_uniq = 0, n_lpr = 0, n_lpv = 0;
+    uint32_t cm = 0;  // largest count appended by this lane (LevelStatus::cmax)
     for (int round = 0;; ++round) {
         int item;
         if (A.granular) {
@@ -1354,13 +1383,16 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
                     const int pos = j ? __popc(s0) + __popc(s1 & lt) : __popc(s0 & lt);
                     A.hub_arena[b0 + pos] = hub[j] | (flg[j] ? kOvfBit : 0u);
                     A.cnt_arena[b0 + pos] = sum[j];
+                    cm = max(cm, count_bound(sum[j], flg[j]));
                 }
                 if (lane == 0) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
             }
         }
         __syncwarp();
     }
+    cm = __reduce_max_sync(FULL, cm);
     if (lane == 0) {
+        if (cm) atomicMax(&A.stt->cmax, cm);
         if (n_uniq) atomicAdd(&A.stt->unique_total, n_uniq);
         if (n_lpr) atomicAdd(&A.stt->lmk_pruned, n_lpr);
         if (n_lpv) atomicAdd(&A.stt->lmk_proven, n_lpv);
@@ -1429,7 +1461,8 @@ cudaError_t launch_dense_prefix(int d, int64_t n, const uint64_t* seg, const uin
 cudaError_t launch_cost(int d, int64_t n, int64_t arcs, const int64_t* rp, const int32_t* col,
                         const int32_t* arc_src, const uint64_t* seg_prev, const uint32_t* hub_arena,
                         const int32_t* hpre, uint32_t* arc_lo, uint32_t* cnt_arc, int64_t* raw_u,
-                        int64_t* lab_size, LevelStatus* stt, int64_t label_limit, int32_t* glist, int32_t* items,
+                        int64_t* lab_size, LevelStatus* stt, int64_t label_limit, const DenseRule& dense,
+                        int32_t* glist, int32_t* items,
                         cudaStream_t st, int64_t* launches) {
     cudaError_t e = cudaMemsetAsync(raw_u, 0, n * 8, st);
     if (e != cudaSuccess) return e;
@@ -1438,9 +1471,10 @@ cudaError_t launch_cost(int d, int64_t n, int64_t arcs, const int64_t* rp, const
                                                                      arc_lo, cnt_arc, (unsigned long long*)raw_u,
                                                                      &stt->prefix_skipped);
     k_cost_vertices<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, rp, seg_prev, raw_u, lab_size, stt, label_limit,
-                                                                  glist);
+                                                                  dense, glist);
     k_bucket_base<<<1, 32, 0, st>>>(stt);
-    k_bucket_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, raw_u, lab_size, stt, label_limit, items);
+    k_bucket_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, rp, raw_u, lab_size, stt, label_limit, dense,
+                                                                items);
     if (launches) *launches += (arcs > 0) + 3;
     return cudaGetLastError();
 }
@@ -1484,6 +1518,19 @@ static void launch_level_nt(int map_kind, bool offchip, int grid, size_t smem_by
         k_level<kMapHash, false, NT><<<grid, NT, smem_bytes, st>>>(A);
     else
         k_level<kMapSeg, false, NT><<<grid, NT, smem_bytes, st>>>(A);
+}
+
+cudaError_t dense_kernel_attrs(int* occupancy) {
+    const size_t bytes = dense_layout().total;
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_level_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bytes);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, (const void*)k_level_dense, kDenseThreads, bytes);
+}
+
+cudaError_t launch_level_dense(int grid, const LevelArgs& A, cudaStream_t st) {
+    k_level_dense<<<grid, kDenseThreads, dense_layout().total, st>>>(A);
+    return cudaGetLastError();
 }
 
 cudaError_t micro_kernel_occupancy(int* occupancy) {

@@ -30,12 +30,36 @@ constexpr size_t kBitmapBudget = 40 * 1024;  // on-chip bytes for the level bitm
 constexpr int kLmkShallow = 32;    // landmarks the filter tests below level kLmkDeepLevel
 constexpr int kLmkDeepLevel = 16;  // from this level on, the filter tests every landmark
 
+// Vertices merged by direct addressing (k_level_dense).
+// Small CTAs: the kernel alternates short phases between barriers, and four
+// CTAs of 256 threads with 11,264-id windows fill each other's gaps better
+// than fewer large ones (R-MAT 2^20 build: 1 x 1024 threads 763 ms, 2 x 512
+// 660 ms, 4 x 256 621 ms, 8 x 128 622 ms but BA 100,000 176 against 171 ms).
+constexpr int kDenseThreads = 256;
+constexpr int kDenseBlocks = 4;             // resident CTAs per SM (53 KB of shared memory each)
+constexpr uint32_t kDenseWindow = 11264;    // ids per on-chip window, a multiple of 128
+constexpr uint32_t kDenseBounds = 1024;     // cells of the table of window starts
+constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (24 MB of slab a CTA)
+constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32 + floor(log2 pulled entries)
+// A vertex with fewer pulled entries cannot overflow the on-chip hash and
+// has too few to pay for the windows: R-MAT 2^20 builds in 615 ms with 2,048
+// here, 643 with 3,500, 677 with 5,000 (R-MAT 65,536 12.9, 13.2, 13.4 ms).
+// Per window of its id range it needs 48 more (window overhead against a
+// hash in device memory): 621 ms with 48, 655 with 96, 743 with 1,024.
+constexpr int64_t kDenseMinRaw = 2048;
+constexpr int64_t kDenseRawPerWindow = 48;
+// Granular builds run one hash CTA per vertex, and the dense kernel at half
+// occupancy: only vertices that would mostly overflow the hash pay (BA
+// 20,011: 7.2 ms, with 2,048 here 7.9 ms).
+constexpr int64_t kDenseMinRawGranular = 16384;
+
 struct LevelStatus {
     unsigned long long raw_total;
     unsigned long long unique_total;
     unsigned long long bump;        // arena fill after this level
     unsigned long long need_cap_c;  // largest candidate table of the off-chip class
     unsigned long long need_cap_u;  // largest label table of the off-chip class
+    unsigned long long need_cap_d;  // most candidates a dense vertex can have
     unsigned long long active_arcs;
     int n_active;
     int n_smem;
@@ -51,6 +75,8 @@ struct LevelStatus {
     int n_giant;     // off-chip vertices whose candidates overflow the slab
     int work_giant;
     int work_micro;
+    int work_dense;
+    unsigned int cmax;  // largest count appended at this level (0xFFFFFFFF: 2^32 or more, or flagged)
     // on-chip attempts and overflows of vertices that can overflow, by
     // floor(log2 pulled entries): where most overflow, the rest go straight
     // to the off-chip pass
@@ -140,6 +166,23 @@ __host__ __device__ inline uint32_t label_cap_for(int64_t lab) {
     return pow2_ceil(want < 64ull ? 64ull : want);
 }
 
+// Which vertices a level merges by direct addressing: `on` for the level,
+// and the largest count of the level below.
+struct DenseRule {
+    int on;
+    uint32_t cmax;
+    int64_t min_raw;
+    const int32_t* comp_base;
+};
+
+// u (id span + first id of its graph) with `raw` pulled entries over deg arcs.
+__host__ __device__ inline bool dense_vertex(const DenseRule& R, int64_t raw, int64_t span, int64_t deg) {
+    const int64_t windows = (span + kDenseWindow - 1) / kDenseWindow;
+    return R.on && raw >= R.min_raw && raw >= kDenseRawPerWindow * windows && raw < ((int64_t)1 << 32) &&
+           (uint64_t)R.cmax * (uint64_t)(deg + 1) < ((uint64_t)1 << 32) &&
+           (raw < span ? raw : span) <= (int64_t)kDenseSlabCap;
+}
+
 enum MapKind { kMapBitmap = 0, kMapHash = 1, kMapSeg = 2 };
 
 // Bytes of the label-map region for a map kind (host plan and kernel must
@@ -185,11 +228,15 @@ cudaError_t launch_dense_prefix(int d, int64_t n, const uint64_t* seg, const uin
 cudaError_t launch_cost(int d, int64_t n, int64_t arcs, const int64_t* rp, const int32_t* col,
                         const int32_t* arc_src, const uint64_t* seg_prev, const uint32_t* hub_arena,
                         const int32_t* hpre, uint32_t* arc_lo, uint32_t* cnt_arc, int64_t* raw_u,
-                        int64_t* lab_size, LevelStatus* stt, int64_t label_limit, int32_t* glist, int32_t* items,
-                        cudaStream_t st, int64_t* launches);
+                        int64_t* lab_size, LevelStatus* stt, int64_t label_limit, const DenseRule& dense,
+                        int32_t* glist, int32_t* items, cudaStream_t st, int64_t* launches);
 cudaError_t level_kernel_attrs(int map_kind, size_t smem_bytes, int* occupancy, int nt = kLevelThreads);
 cudaError_t launch_level(int map_kind, bool offchip, int grid, size_t smem_bytes, const LevelArgs& A,
                          cudaStream_t st, int nt = kLevelThreads);
+// Direct addressing for vertices with many pulled entries (k_level_dense).
+// Per CTA: a slab of A.cap_c_max candidates of 12 bytes in A.gscratch.
+cudaError_t dense_kernel_attrs(int* occupancy);
+cudaError_t launch_level_dense(int grid, const LevelArgs& A, cudaStream_t st);
 // The warp-per-vertex variant for vertices with fewer than 2^kMicroBucket
 // pulled entries (k_level_micro).
 cudaError_t micro_kernel_occupancy(int* occupancy);
