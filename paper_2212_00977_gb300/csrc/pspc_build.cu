@@ -1028,10 +1028,10 @@ struct Builder {
             size_t slab = 0;
             int dense_grid = 0;
             if (n_dense > 0) {
-                // candidate slabs of 12 bytes an entry, one per persistent
+                // candidate slabs of 16 bytes an entry, one per persistent
                 // CTA; granular builds leave half of every SM
                 A.cap_c_max = ((uint32_t)hstt->need_cap_d + 31) & ~31u;
-                slab = (size_t)A.cap_c_max * 12;
+                slab = (size_t)A.cap_c_max * 16;
                 dense_grid = std::min(n_dense, sms * (o.granular ? std::max(1, plan.dense_occupancy / 2) : plan.dense_occupancy));
                 dense_grid = (int)std::min<size_t>(dense_grid, std::max<size_t>(1, ((size_t)4 << 30) / slab));
                 if (o.max_ctas > 0) dense_grid = std::min(dense_grid, o.max_ctas);

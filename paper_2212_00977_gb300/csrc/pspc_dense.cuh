@@ -81,8 +81,8 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
     extern __shared__ __align__(16) uint8_t smem[];
     constexpr int NT = kDenseThreads, kWarps = NT / 32;
     constexpr uint32_t W = kDenseWindow;
-    __shared__ int s_item, s_next, s_kept;
-    __shared__ uint32_t s_lmk[kLmkMax / 2];
+    __shared__ int s_item, s_next, s_lpr, s_lpv, s_open;
+    __shared__ __align__(16) uint32_t s_lmk[kLmkMax / 2];
     __shared__ uint64_t s_useg[kUSideLevels];
     __shared__ int s_wcnt[kWarps];
     __shared__ uint32_t s_wsum[kWarps];
@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
     uint32_t* shub = (uint32_t*)(A.gscratch + (size_t)blockIdx.x * A.gscratch_stride);
     uint32_t* scnt = shub + A.cap_c_max;
     uint32_t* list = scnt + A.cap_c_max;
+    uint32_t* undecided = list + A.cap_c_max;
     uint32_t cm = 0;  // largest count appended by this thread
     uint32_t dirty = W;  // words of the counts' memory to clear for the next vertex
     for (uint32_t i = tid; i < kDenseWords; i += NT) mem[i] = 0u;
@@ -109,6 +110,9 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
         if (tid == 0) {
             s_item = atomicAdd(A.work, 1);
             s_next = 0;
+            s_lpr = 0;
+            s_lpv = 0;
+            s_open = 0;
         }
         for (uint32_t i = tid; i < dirty; i += NT) acc[i] = 0u;
         dirty = 0;
@@ -120,7 +124,8 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
         const int deg = (int)(A.rp[u + 1] - a0);
         const uint32_t span = (uint32_t)u - cbase;  // candidates are cbase + [0, span)
         const uint32_t nwin = (span + W - 1) / W, nb = nwin - 1;
-        if (A.lmk && tid < A.lmk_stride / 4) s_lmk[tid] = __ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + tid);
+        if (A.lmk && tid < A.lmk_stride / 4)
+            s_lmk[tid] = lmk_clamp(__ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + tid));
 
         // Where each window starts in the pulled run of every arc, and in
         // u's own segments of levels d-1 and d-2 (the only ones that a
@@ -268,7 +273,6 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
         // |L_1(u)| arcs of its row) are walked and the ids met marked in a
         // bitmap over the counts' memory, 32 kDenseWindow ids at a time.
         bool listed = false;  // list[] holds the candidates (else all of the slab)
-        int kept = M;
         if (d == 3 && M > 0) {
             const int len1 = (int)seg_len(__ldg(A.seg + n + u));
             const uint32_t from0 = A.hpre ? (uint32_t)__ldg(A.hpre + u) : 0u;  // ids below are members, no candidates
@@ -352,13 +356,15 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
             listed = true;
             for (int c = tid; c < M; c += NT) list[c] = (uint32_t)c;
             __syncthreads();
-            int n_proven = 0;
+            int open = M;
             if (A.lmk) {
-                kept = landmark_filter<NT>(A, s_lmk, d, list, shub, M, s_wcnt, &s_kept, &n_proven);
-                if (tid == 0 && kept < M) atomicAdd(&A.stt->lmk_pruned, (unsigned long long)(M - kept));
-                if (tid == 0 && n_proven) atomicAdd(&A.stt->lmk_proven, (unsigned long long)n_proven);
+                if (A.lmk_words <= 4) landmark_filter<NT, 4>(A, s_lmk, d, list, shub, M, undecided, &s_lpr, &s_lpv, &s_open);
+                else landmark_filter<NT, 8>(A, s_lmk, d, list, shub, M, undecided, &s_lpr, &s_lpv, &s_open);
+                __syncthreads();
+                open = s_open;
+                if (tid == 0 && s_lpr) atomicAdd(&A.stt->lmk_pruned, (unsigned long long)s_lpr);
+                if (tid == 0 && s_lpv) atomicAdd(&A.stt->lmk_proven, (unsigned long long)s_lpv);
             }
-            const int open = kept - n_proven;
             if (open > 0) {
                 SegMap sm;
                 sm.seg = A.seg;
@@ -391,16 +397,16 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
                 const bool useg_on = d - 2 < kUSideLevels;
                 if (useg_on && tid < d - 1) s_useg[tid] = __ldg(A.seg + (int64_t)tid * n + u);
                 __syncthreads();
-                prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, shub, kept, open, &s_next,
-                              useg_on ? s_useg : nullptr, s_wcnt);
+                prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, shub, A.lmk ? undecided : nullptr, M, open,
+                              &s_next, useg_on ? s_useg : nullptr, s_wcnt);
                 __syncthreads();
             }
         }
 
         // 3. survivors, in hub order, appended as L_d(u): each warp owns a
         // run of the candidates
-        const int per = ((kept + kWarps - 1) / kWarps + 31) & ~31;
-        const int c0 = warp * per, c1 = c0 + per < kept ? c0 + per : kept;
+        const int per = ((M + kWarps - 1) / kWarps + 31) & ~31;
+        const int c0 = warp * per, c1 = c0 + per < M ? c0 + per : M;
         int mine = 0;
         for (int c = c0 + lane; c < c1; c += 32) mine += !((listed ? list[c] : shub[c]) & kPrunedBit);
         mine = __reduce_add_sync(0xFFFFFFFFu, mine);

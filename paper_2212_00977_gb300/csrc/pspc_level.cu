@@ -450,7 +450,7 @@ __device__ bool scan_levels(const Map& mp, const uint64_t* __restrict__ seg, con
 template <int G, class Map>
 __device__ void prune_candidates(const Map& mp, const uint64_t* __restrict__ seg,
                                  const uint32_t* __restrict__ hub_arena, int64_t n, int d, uint32_t* list,
-                                 const uint32_t* ckeys, int M, int* next) {
+                                 const uint32_t* ckeys, const uint32_t* open, int M, int* next) {
     auto tile = cg::tiled_partition<G>(cg::this_thread_block());
     const int gl = tile.thread_rank();
     for (;;) {
@@ -458,8 +458,9 @@ __device__ void prune_candidates(const Map& mp, const uint64_t* __restrict__ seg
         if (gl == 0) c = atomicAdd(next, 1);
         c = tile.shfl(c, 0);
         if (c >= M) break;
+        if (open) c = (int)open[c];
         const uint32_t slot = list[c];
-        if (slot & kProvenBit) continue;
+        if (slot & (kProvenBit | kPrunedBit)) continue;
         const uint32_t h = ckeys[slot] & kHubMask;
         const bool pruned = scan_levels<G>(mp, seg, hub_arena, n, d, h, 1, d - 2, nullptr);
         if (pruned && gl == 0) list[c] = slot | kPrunedBit;
@@ -483,13 +484,13 @@ __device__ void prune_split(const Map& mp, const uint64_t* __restrict__ seg, con
     const int groups = kWarps / wpc, g = warp / wpc, j = warp % wpc;
     if (tid < kWarps) s_flag[tid] = 0;
     __syncthreads();
-    // position in list of the g-th candidate that is not proven
+    // position in list of the g-th undecided candidate
     int c = -1;
     if (g < P) {
         int seen = 0;
         for (int base = 0; base < M && c < 0; base += 32) {
             const int i = base + lane;
-            const bool open = i < M && !(list[i] & kProvenBit);
+            const bool open = i < M && !(list[i] & (kProvenBit | kPrunedBit));
             const unsigned bal = __ballot_sync(0xFFFFFFFFu, open);
             const int cnt = __popc(bal);
             if (seen + cnt > g) {
@@ -534,7 +535,7 @@ __device__ __forceinline__ bool seg_contains(const uint32_t* xs, uint32_t len, u
 template <int G, class Map>
 __device__ void prune_by_level(const Map& mp, const uint64_t* __restrict__ seg,
                                const uint32_t* __restrict__ hub_arena, int64_t n, int d, uint32_t* list,
-                               const uint32_t* ckeys, int M, int* next, const uint64_t* useg) {
+                               const uint32_t* ckeys, const uint32_t* open, int M, int* next, const uint64_t* useg) {
     auto tile = cg::tiled_partition<G>(cg::this_thread_block());
     const int gl = tile.thread_rank();
     for (;;) {
@@ -542,8 +543,9 @@ __device__ void prune_by_level(const Map& mp, const uint64_t* __restrict__ seg,
         if (gl == 0) c = atomicAdd(next, 1);
         c = tile.shfl(c, 0);
         if (c >= M) break;
+        if (open) c = (int)open[c];
         const uint32_t slot = list[c];
-        if (slot & kProvenBit) continue;
+        if (slot & (kProvenBit | kPrunedBit)) continue;
         const uint32_t h = ckeys[slot] & kHubMask;
         bool pruned = false;
         for (int k = 1; k <= d - 2 && !pruned; ++k) {
@@ -594,81 +596,103 @@ __device__ void prune_by_level(const Map& mp, const uint64_t* __restrict__ seg,
 // Many candidates: 8 lanes each, level by level (most are pruned within the
 // first entries of L_1(h), so reading further descriptors up front only
 // costs loads). Few candidates: wider groups over the concatenated levels,
-// so that the long scans of deep levels keep all lanes busy.
+// so that the long scans of deep levels keep all lanes busy. open: the
+// positions of the to_scan undecided entries of list[0..M), or NULL (list
+// entries that carry a verdict are skipped).
 template <int NT, class Map>
 __device__ __forceinline__ void prune_all(const Map& mp, const uint64_t* seg, const uint32_t* hub_arena, int64_t n,
-                                          int d, uint32_t* list, const uint32_t* ckeys, int M, int to_scan,
-                                          int* next, const uint64_t* useg, int* s_flag) {
-    if (to_scan >= 64) prune_by_level<8>(mp, seg, hub_arena, n, d, list, ckeys, M, next, useg);
-    else if (to_scan >= NT / 32) prune_candidates<16>(mp, seg, hub_arena, n, d, list, ckeys, M, next);
+                                          int d, uint32_t* list, const uint32_t* ckeys, const uint32_t* open, int M,
+                                          int to_scan, int* next, const uint64_t* useg, int* s_flag) {
+    const int items = open ? to_scan : M;
+    if (to_scan >= 64) prune_by_level<8>(mp, seg, hub_arena, n, d, list, ckeys, open, items, next, useg);
+    else if (to_scan >= NT / 32) prune_candidates<16>(mp, seg, hub_arena, n, d, list, ckeys, open, items, next);
     else prune_split<NT>(mp, seg, hub_arena, n, d, list, ckeys, M, to_scan, s_flag);
 }
 
 // Landmark filter (Section "Landmark-Based Filtering"). For a candidate h
 // of u at level d, rule 2 prunes h exactly when sd(u,h) < d. Each landmark
 // l bounds sd(u,h) from both sides: sd(u,h) <= sd(u,l) + sd(l,h), and
-// sd(u,h) >= |sd(u,l) - sd(l,h)|. An upper bound below d prunes h at once;
-// a lower bound of at least d proves that h survives (it keeps its list
-// entry, marked kProvenBit, and skips the label scan). Distances are uint16
-// (0xFFFF = unknown): the sum is taken with saturation and compared with d
-// (at most 32767), so an unknown or saturated sum never prunes, and 0xFFFF
-// on either side gives no lower bound. The candidates not pruned are
-// compacted to list[0..kept) in the same order (in rounds of one candidate
-// per thread: every read of a round precedes its writes, and no write
-// reaches past the round's reads). Returns kept; *n_proven receives the
-// proven ones among them.
-template <int NT>
-__device__ int landmark_filter(const LevelArgs& A, const uint32_t* s_lmk, int d, uint32_t* list,
-                               const uint32_t* ckeys, int M, int* s_wcnt, int* s_kept, int* n_proven) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t dd = (uint32_t)d * 0x00010001u;  // d <= 32767 in both halfwords
-    const int words = A.lmk_words;
-    int kept = 0, proven = 0;
-    for (int base = 0; base < M; base += NT) {
-        const int c = base + tid;
-        uint32_t slot = 0;
-        bool keep = false, sure = false;
-        if (c < M) {
-            slot = list[c];
-            const uint4* row = (const uint4*)(A.lmk + (size_t)(ckeys[slot] & kHubMask) * A.lmk_stride);
-            uint32_t hit = 0, far = 0;
-            // two uint16 distances per word; 0xFFFF (undefined) saturates
-            // the sum and is masked out of the difference test
+// sd(u,h) >= |sd(u,l) - sd(l,h)|. An upper bound below d prunes h at once
+// (kPrunedBit); a lower bound of at least d proves that h survives
+// (kProvenBit). Distances are uint16, 0xFFFF where undefined, and are
+// clamped to 32,767 here: d is at most that, so a clamped value never prunes
+// and only lowers the lower bound, and u and its candidate h are connected,
+// so a landmark is undefined for both (difference 0) or for neither.
+//
+// G lanes take a candidate and read its row 16 bytes a lane, so a warp's load
+// covers whole rows (a thread per candidate read 32 rows at 32 places), and
+// a word of two distances costs a clamp and three fused add-and-min/max
+// instructions (the saturating and comparing SIMD intrinsics it replaces
+// expand to some forty). On grid 256x256 the filter took 36% of the light
+// kernel's cycles.
+constexpr uint32_t kLmkClamp = 0x7FFF7FFFu;
+
+__device__ __forceinline__ uint32_t lmk_clamp(uint32_t x) { return __vminu2(x, kLmkClamp); }
+
+// Bit 0: h is pruned, bit 1: h is proven (the same in all G lanes of the
+// group, which act together). ua: u's row, clamped, on chip.
+template <int G>
+__device__ __forceinline__ uint32_t landmark_verdict(const uint32_t* ua, const uint8_t* row, int words, int d, int gl,
+                                                     unsigned group) {
+    uint32_t up = kLmkClamp;                   // smallest sum
+    uint32_t hi = 0x80008000u, lo = kLmkClamp;  // largest and smallest sd(l,h) - sd(u,l) - 1
+    for (int w = gl; w < words; w += G) {
+        const uint4 b4 = __ldg((const uint4*)row + w);
+        const uint4 a4 = ((const uint4*)ua)[w];
+        const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w}, aw[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
-            for (int w = 0; w < kLmkMax / 8; ++w)
-                if (w < words) {
-                    const uint4 b4 = __ldg(row + w);
-                    const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint32_t a = s_lmk[4 * w + q], b = bw[q];
-                        hit |= __vcmpltu2(__vaddus2(a, b), dd);
-                        const uint32_t known = ~(__vcmpeq2(a, 0xFFFFFFFFu) | __vcmpeq2(b, 0xFFFFFFFFu));
-                        far |= __vcmpgeu2(__vabsdiffu2(a, b), dd) & known;
-                    }
-                }
-            keep = hit == 0u;
-            sure = keep && far != 0u;
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t b = lmk_clamp(bw[q]);
+            up = __viaddmin_u16x2(aw[q], b, up);
+            hi = __viaddmax_s16x2(b, ~aw[q], hi);
+            lo = __viaddmin_s16x2(b, ~aw[q], lo);
         }
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
-        const unsigned bsure = __ballot_sync(0xFFFFFFFFu, sure);
-        if (lane == 0) s_wcnt[warp] = __popc(bal) | (__popc(bsure) << 16);
-        __syncthreads();
-        int before = 0, round = 0, round_sure = 0;
-        for (int w = 0; w < NT / 32; ++w) {
-            const int v = s_wcnt[w];
-            before += w < warp ? (v & 0xFFFF) : 0;
-            round += v & 0xFFFF;
-            round_sure += v >> 16;
-        }
-        if (keep) list[kept + before + __popc(bal & ((1u << lane) - 1u))] = slot | (sure ? kProvenBit : 0u);
-        kept += round;
-        proven += round_sure;
-        __syncthreads();
     }
-    if (tid == 0) *s_kept = kept;
-    *n_proven = proven;
-    return kept;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        up = __vminu2(up, __shfl_xor_sync(group, up, o, G));
+        hi = __vmaxs2(hi, __shfl_xor_sync(group, hi, o, G));
+        lo = __vmins2(lo, __shfl_xor_sync(group, lo, o, G));
+    }
+    const int sum = min((int)(up & 0xFFFFu), (int)(up >> 16));
+    const int over = max((int)(int16_t)(hi & 0xFFFFu), (int)(int16_t)(hi >> 16)) + 1;
+    const int under = min((int)(int16_t)(lo & 0xFFFFu), (int)(int16_t)(lo >> 16)) + 1;
+    return (sum < d ? 1u : 0u) | ((over >= d || under <= -d) ? 2u : 0u);
+}
+
+// The filter over list[0..M): the verdict is added to each entry, and the
+// undecided positions are collected in open[0..*s_open) (any order) when
+// open is given. *s_pruned, *s_proven and *s_open (zero before) receive the
+// counts; the caller's barrier follows.
+template <int NT, int G>
+__device__ void landmark_filter(const LevelArgs& A, const uint32_t* ua, int d, uint32_t* list, const uint32_t* ckeys,
+                                int M, uint32_t* open, int* s_pruned, int* s_proven, int* s_open) {
+    const int tid = threadIdx.x, lane = tid & 31, gl = lane % G;
+    constexpr int kPerWarp = 32 / G, kStep = NT / G;
+    int pruned = 0, proven = 0;
+    for (int base = tid / 32 * kPerWarp; base < M; base += kStep) {  // warp-uniform
+        const int c = base + lane / G;
+        uint32_t slot = 0, v = 1u;
+        if (c < M) slot = list[c];
+        const uint32_t h = c < M ? ckeys[slot] & kHubMask : 0u;
+        v = landmark_verdict<G>(ua, A.lmk + (size_t)h * A.lmk_stride, c < M ? A.lmk_words : 0, d, gl, 0xFFFFFFFFu);
+        const bool lead = gl == 0 && c < M;
+        const bool is_open = lead && v == 0u;
+        if (lead && v) list[c] = slot | (v & 1u ? kPrunedBit : kProvenBit);
+        pruned += lead && (v & 1u);
+        proven += lead && v == 2u;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, is_open);
+        if (m) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(s_open, __popc(m));
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+            if (open && is_open) open[at + __popc(m & ((1u << lane) - 1u))] = (uint32_t)c;
+        }
+    }
+    pruned = __reduce_add_sync(0xFFFFFFFFu, pruned);
+    proven = __reduce_add_sync(0xFFFFFFFFu, proven);
+    if (lane == 0 && pruned) atomicAdd(s_pruned, pruned);
+    if (lane == 0 && proven) atomicAdd(s_proven, proven);
 }
 
 __device__ void block_bitonic_sort(unsigned long long* buf, uint32_t P) {
@@ -695,8 +719,9 @@ __device__ void block_bitonic_sort(unsigned long long* buf, uint32_t P) {
 template <int kMap, bool kOffChip, int NT>
 __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelArgs A) {
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ int s_item, s_nkeys, s_abort, s_m, s_next, s_nsurv, s_kept, s_route;
-    __shared__ uint32_t s_lmk[kLmkMax / 2];  // u's landmark distances (uint16 pairs)
+    __shared__ int s_item, s_nkeys, s_abort, s_m, s_next, s_nsurv, s_route;
+    __shared__ int s_lpr, s_lpv, s_open;             // the landmark filter's counts
+    __shared__ __align__(16) uint32_t s_lmk[kLmkMax / 2];  // u's landmark distances (uint16 pairs, clamped)
     __shared__ uint64_t s_useg[kUSideLevels];  // u's level descriptors for the rule-2 scan
     __shared__ int s_wcnt[NT / 32];
     __shared__ unsigned long long s_base;
@@ -799,8 +824,12 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
             s_m = 0;
             s_next = 0;
             s_nsurv = 0;
+            s_lpr = 0;
+            s_lpv = 0;
+            s_open = 0;
         }
-        if (A.lmk && tid < A.lmk_stride / 4) s_lmk[tid] = __ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + tid);
+        if (A.lmk && tid < A.lmk_stride / 4)
+            s_lmk[tid] = lmk_clamp(__ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + tid));
         __syncthreads();
 
         // 1. label map of L_<d(u)
@@ -948,7 +977,7 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         for (uint32_t slot = tid; slot < cap_c; slot += NT)
             if (ckeys[slot] != kEmpty) list[atomicAdd(&s_m, 1)] = slot;
         __syncthreads();
-        int M = s_m;
+        const int M = s_m;
 
         // 3a. d = 3: rule 2 asks for a common neighbour x of u and h ranked
         // above h (x in L_1(u) and x in L_1(h)). Walk, for every x in L_1(u),
@@ -1032,14 +1061,16 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         }
 
         // 3. prune rule 2 over levels 1..d-2 of each candidate's label
-        int M_scan = M, n_proven = 0;
+        int ns = M;  // candidates left to scan
         if (d >= 3 && !marked && M > 0 && A.lmk) {
-            M_scan = landmark_filter<NT>(A, s_lmk, d, list, ckeys, M, s_wcnt, &s_kept, &n_proven);
-            if (tid == 0 && M_scan < M) atomicAdd(&A.stt->lmk_pruned, (unsigned long long)(M - M_scan));
-            if (tid == 0 && n_proven) atomicAdd(&A.stt->lmk_proven, (unsigned long long)n_proven);
+            if (A.lmk_words <= 4) landmark_filter<NT, 4>(A, s_lmk, d, list, ckeys, M, nullptr, &s_lpr, &s_lpv, &s_open);
+            else landmark_filter<NT, 8>(A, s_lmk, d, list, ckeys, M, nullptr, &s_lpr, &s_lpv, &s_open);
+            __syncthreads();
+            ns = s_open;
+            if (tid == 0 && s_lpr) atomicAdd(&A.stt->lmk_pruned, (unsigned long long)s_lpr);
+            if (tid == 0 && s_lpv) atomicAdd(&A.stt->lmk_proven, (unsigned long long)s_lpv);
         }
-        if (d >= 3 && !marked && M_scan > n_proven) {
-            const int ns = M_scan - n_proven;
+        if (d >= 3 && !marked && ns > 0) {
             // u's level descriptors, for scanning u's side when it is shorter
             // (not with bitmaps: their probes cost one on-chip read)
             const bool useg_on = kMap != kMapBitmap && d - 2 < kUSideLevels;
@@ -1047,14 +1078,12 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
             __syncthreads();
             const uint64_t* useg = useg_on ? s_useg : nullptr;
             if constexpr (kMap == kMapBitmap)
-                prune_all<NT>(bm, A.seg, A.hub_arena, n, d, list, ckeys, M_scan, ns, &s_next, useg, s_wcnt);
+                prune_all<NT>(bm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt);
             else if constexpr (kMap == kMapHash)
-                prune_all<NT>(hm, A.seg, A.hub_arena, n, d, list, ckeys, M_scan, ns, &s_next, useg, s_wcnt);
-            else prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, ckeys, M_scan, ns, &s_next, useg, s_wcnt);
+                prune_all<NT>(hm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt);
+            else prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt);
             __syncthreads();
         }
-        M = M_scan;  // list[0..M) now holds every candidate that can survive
-
         // 4. survivors, hub-sorted, appended as L_d(u). Candidate hubs are < u:
         // when a bitmap of u bits and its word prefix fit the map region, a
         // survivor's rank is the prefix of its word plus a popcount; else a
@@ -1167,7 +1196,7 @@ __device__ __forceinline__ void add_count(uint64_t& sum, uint32_t& flag, uint64_
 __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A) {
     __shared__ uint32_t s_hub[kMicroWarps][64];
     __shared__ unsigned long long s_cnt[kMicroWarps][64];
-    __shared__ uint32_t s_lmkw[kMicroWarps][kLmkMax / 2];
+    __shared__ __align__(16) uint32_t s_lmkw[kMicroWarps][kLmkMax / 2];
     const unsigned FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int d = A.d;
@@ -1324,30 +1353,32 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
         if (d >= 3 && uniq > 0) {
             bool und[2] = {cand[0], cand[1]};
             if (A.lmk) {
-                for (int i = lane; i < A.lmk_stride / 4; i += 32) ul[i] = __ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + i);
+                for (int i = lane; i < A.lmk_stride / 4; i += 32)
+                    ul[i] = lmk_clamp(__ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + i));
+                // the candidates' hubs in order (the staged entries are done
+                // with), eight lanes to each, then the verdicts back
+                const unsigned c0 = __ballot_sync(FULL, cand[0]), c1 = __ballot_sync(FULL, cand[1]);
+                const int at[2] = {__popc(c0 & lt), __popc(c0) + __popc(c1 & lt)};
+                uint32_t* verdict = (uint32_t*)cbuf;
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    if (cand[j]) hb[at[j]] = hub[j];
                 __syncwarp();
-                const uint32_t dd = (uint32_t)d * 0x00010001u;
+                for (int base = 0; base < uniq; base += 4) {
+                    const int c = base + lane / 8;
+                    const uint32_t v = landmark_verdict<8>(ul, A.lmk + (size_t)(c < uniq ? hb[c] : 0u) * A.lmk_stride,
+                                                           c < uniq ? A.lmk_words : 0, d, lane % 8, FULL);
+                    if (c < uniq && lane % 8 == 0) verdict[c] = v;
+                }
+                __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    if (!cand[j]) continue;
-                    const uint4* row = (const uint4*)(A.lmk + (size_t)hub[j] * A.lmk_stride);
-                    uint32_t hit = 0, far = 0;
-                    for (int q4 = 0; q4 < A.lmk_words; ++q4) {
-                        const uint4 b4 = __ldg(row + q4);
-                        const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint32_t a = ul[4 * q4 + q], b = bw[q];
-                            hit |= __vcmpltu2(__vaddus2(a, b), dd);
-                            const uint32_t known = ~(__vcmpeq2(a, 0xFFFFFFFFu) | __vcmpeq2(b, 0xFFFFFFFFu));
-                            far |= __vcmpgeu2(__vabsdiffu2(a, b), dd) & known;
-                        }
-                    }
-                    if (hit) {
+                    const uint32_t v = cand[j] ? verdict[at[j]] : 0u;
+                    if (v & 1u) {
                         surv[j] = false;
                         und[j] = false;
                         ++n_lpr;
-                    } else if (far) {
+                    } else if (v & 2u) {
                         und[j] = false;
                         ++n_lpv;
                     }
@@ -1391,6 +1422,11 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
         __syncwarp();
     }
     cm = __reduce_max_sync(FULL, cm);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {  // the verdicts were counted by the candidates' lanes
+        n_lpr += __shfl_xor_sync(FULL, n_lpr, o);
+        n_lpv += __shfl_xor_sync(FULL, n_lpv, o);
+    }
     if (lane == 0) {
         if (cm) atomicMax(&A.stt->cmax, cm);
         if (n_uniq) atomicAdd(&A.stt->unique_total, n_uniq);

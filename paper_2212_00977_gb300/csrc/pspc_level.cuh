@@ -39,7 +39,7 @@ constexpr int kDenseThreads = 256;
 constexpr int kDenseBlocks = 4;             // resident CTAs per SM (53 KB of shared memory each)
 constexpr uint32_t kDenseWindow = 11264;    // ids per on-chip window, a multiple of 128
 constexpr uint32_t kDenseBounds = 1024;     // cells of the table of window starts
-constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (24 MB of slab a CTA)
+constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (32 MB of slab a CTA)
 constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32 + floor(log2 pulled entries)
 // A vertex with fewer pulled entries cannot overflow the on-chip hash and
 // has too few to pay for the windows: R-MAT 2^20 builds in 615 ms with 2,048
@@ -234,7 +234,7 @@ cudaError_t level_kernel_attrs(int map_kind, size_t smem_bytes, int* occupancy, 
 cudaError_t launch_level(int map_kind, bool offchip, int grid, size_t smem_bytes, const LevelArgs& A,
                          cudaStream_t st, int nt = kLevelThreads);
 // Direct addressing for vertices with many pulled entries (k_level_dense).
-// Per CTA: a slab of A.cap_c_max candidates of 12 bytes in A.gscratch.
+// Per CTA: a slab of A.cap_c_max candidates of 16 bytes in A.gscratch.
 cudaError_t dense_kernel_attrs(int* occupancy);
 cudaError_t launch_level_dense(int grid, const LevelArgs& A, cudaStream_t st);
 // The warp-per-vertex variant for vertices with fewer than 2^kMicroBucket
