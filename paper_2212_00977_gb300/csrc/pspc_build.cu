@@ -998,7 +998,7 @@ struct Builder {
         A.stt = stt;
         A.retry_list = glist + hstt->n_global;
         A.comp_base = comp_base;
-        A.lmk = out.lmk;
+        A.lmk = d <= kMaxDist ? out.lmk : nullptr;  // the filter compares 15-bit distances
         A.lmk_stride = out.lmk_stride;
         // shallow levels test the first kLmkShallow landmarks only: their
         // short distances seldom prove survival, and half the row is read
