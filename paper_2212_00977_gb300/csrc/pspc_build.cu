@@ -602,7 +602,10 @@ struct LevelPlan {
     int occupancy = 0;
     size_t light_smem_bytes = 0;  // light vertices: kLightThreads CTAs, segment-search map
     int light_occupancy = 0;
-    int micro_occupancy = 0;      // tiny vertices: the warp-per-vertex kernel
+    int micro_occupancy = 0;      // small vertices: the warp-per-vertex kernel
+    int tiny_occupancy = 0;       // and its narrower form
+    int prove_occupancy = 0;      // the deferred scans: the neighbours' proof,
+    int scan_occupancy = 0;       // and the scan
     int dense_occupancy = 0;      // many pulled entries: direct addressing (0: not used)
 };
 
@@ -644,6 +647,9 @@ struct Builder {
     int64_t* raw_u = nullptr;
     int64_t* lab_size = nullptr;
     int32_t* items = nullptr;
+    HeldSegment* held = nullptr;     // deferred scans: one segment per vertex at most, and the queue
+    DeferredScan* scans = nullptr;   // (and behind it the scans left after the proof)
+    unsigned int scan_cap = 0;
     int32_t* glist = nullptr;
     LevelStatus* stt = nullptr;
     LevelStatus hs;               // host copy of the level status
@@ -679,6 +685,8 @@ struct Builder {
         dfree(raw_u, st);
         dfree(lab_size, st);
         dfree(items, st);
+        dfree(held, st);
+        dfree(scans, st);
         dfree(glist, st);
         dfree(stt, st);
         dfree(err, st);
@@ -1003,27 +1011,38 @@ struct Builder {
         // shallow levels test the first kLmkShallow landmarks only: their
         // short distances seldom prove survival, and half the row is read
         A.lmk_words = d < kLmkDeepLevel ? std::min(out.lmk_stride / 16, 2 * kLmkShallow / 16) : out.lmk_stride / 16;
+        if (d >= kDeferLevel && A.lmk && (int64_t)hstt->n_active * d >= kDeferWork) {
+            if (!held) {
+                scan_cap = (unsigned)std::min<int64_t>(std::max<int64_t>(4 * n, 1 << 16), 1 << 26);
+                PSPC_TRY_CUDA(dalloc(&held, n, st));
+                PSPC_TRY_CUDA(dalloc(&scans, 2 * (size_t)scan_cap, st));
+            }
+            A.held = held;
+            A.scans = scans;
+            A.scan_cap = scan_cap;
+        }
         if (hstt->n_smem > 0) {
             // Items are bucketed heaviest first. Light vertices (fewer than
             // 2^kLightBucket pulled entries) run in small CTAs with small
             // tables and the segment-search map, so that many of them share
             // an SM; the others in full-size CTAs.
-            int n_light = 0, n_micro = 0;
-            // Automatic: one warp per tiny vertex at levels 2 and 3, and
-            // deeper (up to level 127) while the last level had few
-            // candidates per vertex: there the warp's own rule-2 scans are
-            // short or rare.
+            int n_light = 0, n_micro = 0, n_tiny = 0;
+            // Automatic: one warp per small vertex at levels 2 and 3, and
+            // deeper while the last level had few candidates per vertex:
+            // there the warp's own rule-2 scans are short or rare.
             bool warp_level = o.warp_levels > 0 && d <= o.warp_levels;
             if (o.warp_levels == 0 && !out.lstats.empty()) {
                 const pspc_level_stat_t& pl = out.lstats.back();
-                warp_level = d <= 3 || (d <= kWarpLevelsMax && pl.active_vertices > 0 &&
+                warp_level = d <= 3 || (pl.active_vertices > 0 &&
                                         pl.unique_candidates < kWarpLevelsFew * pl.active_vertices);
             }
             for (int b = 0; b < kLightBucket; ++b)
-                (warp_level && b < kMicroBucket ? n_micro : n_light) += hstt->bucket_cnt[b];
+                (!warp_level || b >= (d <= 3 ? kTinyBucket : kMicroBucket) ? n_light
+                 : b >= kTinyBucket                                        ? n_micro
+                                                                           : n_tiny) += hstt->bucket_cnt[b];
             int n_dense = 0;
             for (int b = kDenseBucket; b < kBuckets; ++b) n_dense += hstt->bucket_cnt[b];
-            const int n_heavy = hstt->n_smem - n_light - n_micro - n_dense;
+            const int n_heavy = hstt->n_smem - n_light - n_micro - n_tiny - n_dense;
             A.granular = o.granular ? 1 : 0;
             size_t slab = 0;
             int dense_grid = 0;
@@ -1075,20 +1094,32 @@ struct Builder {
                 e = launch_level(kMapSeg, false, grid, plan.light_smem_bytes, A, st, kLightThreads);
                 out.launches += 1;
             }
-            if (e == cudaSuccess && n_micro > 0) {  // one warp per vertex
-                A.items = items + n_dense + n_heavy + n_light;
-                A.n_items = n_micro;
-                A.work = &stt->work_micro;
+            for (int tiny = 0; tiny < 2; ++tiny) {  // one warp per vertex
+                const int count = tiny ? n_tiny : n_micro;
+                if (e != cudaSuccess || count == 0) continue;
+                A.items = items + n_dense + n_heavy + n_light + (tiny ? n_micro : 0);
+                A.n_items = count;
+                A.work = tiny ? &stt->work_tiny : &stt->work_micro;
                 const int per_cta = kMicroThreads / 32;
-                int grid = (n_micro + per_cta - 1) / per_cta;
-                if (!o.granular) grid = std::min(grid, sms * plan.micro_occupancy);
+                int grid = (count + per_cta - 1) / per_cta;
+                if (!o.granular) grid = std::min(grid, sms * (tiny ? plan.tiny_occupancy : plan.micro_occupancy));
                 if (o.max_ctas > 0 && !o.granular) grid = std::min(grid, o.max_ctas);
-                e = launch_level_micro(grid, A, st);
+                e = launch_level_micro(tiny ? 2 : 4, grid, A, st);
                 out.launches += 1;
+            }
+            if (e == cudaSuccess && A.held) {
+                // granular builds leave half of every SM
+                int pg = sms * (o.granular ? std::max(1, plan.prove_occupancy / 2) : plan.prove_occupancy);
+                int sg = sms * (o.granular ? std::max(1, plan.scan_occupancy / 2) : plan.scan_occupancy);
+                if (o.max_ctas > 0) pg = std::min(pg, o.max_ctas);
+                if (o.max_ctas > 0) sg = std::min(sg, o.max_ctas);
+                e = launch_scan_deferred(pg, sg, A, st);
+                out.launches += 2;
             }
             cudaEventRecord(ek1, st);
             PSPC_TRY_CUDA(e);
         }
+        A.held = nullptr;  // off chip the scans run in place
         int rc = read_status();
         if (rc) return rc;
         if (hstt->n_smem > 0) {
@@ -1174,8 +1205,13 @@ struct Builder {
         plan.light_smem_bytes = level_layout(kLightCap, level_map_bytes(kMapSeg, d, 0, 0), kLightThreads).total;
         PSPC_TRY_CUDA(level_kernel_attrs(kMapSeg, plan.light_smem_bytes, &plan.light_occupancy, kLightThreads));
         if (plan.light_occupancy < 1) return PSPC_E_INVAL;
-        PSPC_TRY_CUDA(micro_kernel_occupancy(&plan.micro_occupancy));
-        if (plan.micro_occupancy < 1) return PSPC_E_INVAL;
+        if (plan.micro_occupancy == 0) {  // the same for every level
+            PSPC_TRY_CUDA(micro_kernel_occupancy(4, &plan.micro_occupancy));
+            PSPC_TRY_CUDA(micro_kernel_occupancy(2, &plan.tiny_occupancy));
+            PSPC_TRY_CUDA(scan_kernel_occupancy(&plan.prove_occupancy, &plan.scan_occupancy));
+        }
+        if (plan.micro_occupancy < 1 || plan.tiny_occupancy < 1 || plan.prove_occupancy < 1 ||
+            plan.scan_occupancy < 1) return PSPC_E_INVAL;
         // Direct addressing with the automatic tables only: a caller that
         // asks for smaller ones, a map kind or the push buckets gets the
         // hash kernels.
@@ -1359,7 +1395,11 @@ struct Builder {
                 keep.n_retry = 0;
                 keep.arena_overflow = 0;
                 keep.work_smem = keep.work_global = keep.work_light = keep.work_giant = keep.work_micro = 0;
-                keep.work_dense = 0;
+                keep.work_dense = keep.work_tiny = keep.work_scan = 0;
+                keep.n_held = 0;
+                keep.n_scan = 0;
+                keep.n_scan_open = 0;
+                keep.dropped = 0;
                 keep.cmax = 0;
                 keep.n_giant = 0;
                 memset(keep.route_att, 0, sizeof(keep.route_att));  // the level is re-run from scratch
@@ -1370,7 +1410,7 @@ struct Builder {
             if (rc) break;
             cudaEventRecord(e1, st);
             bump = hstt->bump;
-            const long long added = (long long)(bump - lvl_base[d]);
+            const long long added = (long long)(bump - lvl_base[d] - hstt->dropped);
             float ms = 0.f;
             cudaEventSynchronize(e1);
             cudaEventElapsedTime(&ms, e0, e1);

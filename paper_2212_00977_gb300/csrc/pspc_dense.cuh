@@ -393,12 +393,14 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
                     dirty = (uint32_t)(d - 1) * cw;
                     sm.cache = acc;
                     sm.cwords = cw;
+                } else {
+                    dirty = kWarps * (kDeepFilter + kScanHits);  // the split scan's filters
                 }
                 const bool useg_on = d - 2 < kUSideLevels;
                 if (useg_on && tid < d - 1) s_useg[tid] = __ldg(A.seg + (int64_t)tid * n + u);
                 __syncthreads();
                 prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, shub, A.lmk ? undecided : nullptr, M, open,
-                              &s_next, useg_on ? s_useg : nullptr, s_wcnt);
+                              &s_next, useg_on ? s_useg : nullptr, s_wcnt, sm.cache ? nullptr : acc, u);
                 __syncthreads();
             }
         }

@@ -445,6 +445,149 @@ __device__ bool scan_levels(const Map& mp, const uint64_t* __restrict__ seg, con
     return pruned;
 }
 
+// Rule 2 over levels klo..khi of L(h) against u's label, by one warp and
+// without a map of u. A witness x of L_k(h) lies in L_l(u) with l = d-1-k or
+// d-2-k (see SegMap), so 31 levels of h meet 32 levels of u. The (hub, level)
+// pairs of h set bits of a filter on chip, u's entries probe it for their two
+// levels, and the few that find a bit are looked up in L_k(h) together, a
+// match to a lane. What bounds it is the latency of loads that miss L2 (the
+// labels of a large index do not fit): a search of u's segments for each entry
+// of h was a chain of ten of them, here a step of 31 levels has two, the
+// descriptors and then both labels' entries, kScanUnroll rows of each in
+// flight, and the next step's descriptors are read meanwhile. Returns whether
+// a witness was found (or, then possibly false, *stop was set).
+// mem: `words` words of filter (a power of two), then kScanHits of matches.
+constexpr int kScanUnroll = 4;          // rows of 32 entries in flight
+constexpr uint32_t kScanHits = 64;      // matches kept until they are looked up
+constexpr uint32_t kMicroFilter = 256;  // filter words per warp of the warp-per-vertex kernel,
+constexpr uint32_t kDeepFilter = 256;   // of the light kernel's deep form,
+constexpr uint32_t kScanFilter = 1024;  // and of the deferred scans
+
+__device__ bool scan_filtered(uint32_t* mem, uint32_t words, const uint64_t* __restrict__ seg,
+                              const uint32_t* __restrict__ hub_arena, int64_t n, int64_t u, int d, uint32_t h, int klo,
+                              int khi, const int* stop) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t* filter = mem;
+    uint32_t* hits = mem + words;
+    const int shift = __clz(words) - 4;  // a hash's top bits: 32 per word
+    auto bit_of = [&](uint32_t x, int j) { return (x * 0x9E3779B1u + (uint32_t)j * 0x85EBCA6Bu) >> shift; };
+    // segment of entry i of the concatenated segments: the last lane whose
+    // exclusive prefix is at most i
+    auto locate = [&](uint32_t excl, uint32_t i) {
+        int j = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const uint32_t e = __shfl_sync(FULL, excl, j + step);
+            if (e <= i) j += step;
+        }
+        return j;
+    };
+    auto seg_h = [&](int k0) { return lane < 31 && k0 + lane <= khi ? __ldg(seg + (int64_t)(k0 + lane) * n + h) : 0ull; };
+    auto seg_u = [&](int k0) {
+        const int k = k0 + lane, l = d - 1 - k;
+        return l >= 1 && k <= khi + 1 ? __ldg(seg + (int64_t)l * n + u) : 0ull;
+    };
+    uint64_t sa = seg_h(klo), sb = seg_u(klo);
+    for (int k0 = klo; k0 <= khi; k0 += 31) {
+        const uint64_t ca = sa, cb = sb;
+        if (k0 + 31 <= khi) {
+            sa = seg_h(k0 + 31);
+            sb = seg_u(k0 + 31);
+        }
+        uint32_t ia = seg_len(ca), ib = seg_len(cb);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t ta = __shfl_up_sync(FULL, ia, o), tb = __shfl_up_sync(FULL, ib, o);
+            if (lane >= o) {
+                ia += ta;
+                ib += tb;
+            }
+        }
+        const uint32_t ea = ia - seg_len(ca), eb = ib - seg_len(cb);
+        const uint32_t na = __shfl_sync(FULL, ia, 31), nb = __shfl_sync(FULL, ib, 31);
+        if (na == 0 || nb == 0) continue;
+        const uint64_t pa = seg_start(ca) - ea, pb = seg_start(cb) - eb;
+        // entry word: hub | lane of its segment << 24; kEmpty for none
+        auto load_rows = [&](uint32_t (&x)[kScanUnroll], uint32_t b, uint32_t end, uint32_t excl, uint64_t base) {
+            int j[kScanUnroll];
+#pragma unroll
+            for (int t = 0; t < kScanUnroll; ++t) {
+                x[t] = kEmpty;
+                j[t] = 0;
+                if (b + t * 32 >= end) continue;  // warp-uniform
+                const uint32_t i = b + t * 32 + lane;
+                j[t] = locate(excl, i);
+                const uint64_t pj = __shfl_sync(FULL, base, j[t]);
+                if (i < end) x[t] = __ldg(hub_arena + pj + i);
+            }
+#pragma unroll
+            for (int t = 0; t < kScanUnroll; ++t)
+                if (b + t * 32 + lane < end) x[t] = (x[t] & kHubMask) | (uint32_t)j[t] << 24;
+        };
+        uint32_t xb[kScanUnroll];
+        load_rows(xb, 0, nb, eb, pb);
+        for (uint32_t i = lane; i < words / 4; i += 32) ((uint4*)filter)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+        for (uint32_t b = 0; b < na; b += 32 * kScanUnroll) {
+            uint32_t xa[kScanUnroll];
+            load_rows(xa, b, na, ea, pa);
+#pragma unroll
+            for (int t = 0; t < kScanUnroll; ++t)
+                if (xa[t] != kEmpty) {
+                    const uint32_t bit = bit_of(xa[t] & kHubMask, (int)(xa[t] >> 24));
+                    atomicOr(&filter[bit >> 5], 1u << (bit & 31));
+                }
+        }
+        __syncwarp();
+        int nh = 0;  // matches kept
+        bool found = false, halt = false;
+        auto look_up = [&]() {  // the first 32 kept matches, one to a lane
+            __syncwarp();
+            bool hit = false;
+            if (lane < nh) {
+                const uint32_t x = hits[lane] & kHubMask;
+                const uint64_t s = __ldg(seg + (int64_t)(k0 + (int)(hits[lane] >> 24)) * n + h);
+                const uint32_t at = seg_lower_bound(hub_arena + seg_start(s), seg_len(s), x);
+                hit = at < seg_len(s) && (__ldg(hub_arena + seg_start(s) + at) & kHubMask) == x;
+            }
+            found = __any_sync(FULL, hit);
+            const uint32_t tail = lane + 32 < nh ? hits[lane + 32] : 0u;
+            __syncwarp();
+            if (lane + 32 < nh) hits[lane] = tail;
+            nh = nh > 32 ? nh - 32 : 0;
+        };
+        for (uint32_t b = 0; b < nb && !found && !halt; b += 32 * kScanUnroll) {
+            if (b) load_rows(xb, b, nb, eb, pb);
+#pragma unroll
+            for (int t = 0; t < kScanUnroll; ++t) {
+                if (b + t * 32 >= nb || found) continue;  // warp-uniform
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {  // x at level l of u: levels d-1-l and d-2-l of h
+                    const int jj = (int)(xb[t] >> 24) - o;
+                    bool maybe = false;
+                    if (xb[t] != kEmpty && jj >= 0 && jj < 31) {
+                        const uint32_t bit = bit_of(xb[t] & kHubMask, jj);
+                        maybe = (filter[bit >> 5] >> (bit & 31)) & 1u;
+                    }
+                    const unsigned m = __ballot_sync(FULL, maybe);
+                    if (!m) continue;
+                    if (maybe) hits[nh + __popc(m & lt)] = (xb[t] & kHubMask) | (uint32_t)jj << 24;
+                    nh += __popc(m);
+                    if (nh > 32) look_up();
+                }
+            }
+            if (stop) halt = __any_sync(FULL, *(volatile const int*)stop != 0);
+        }
+        if (nh > 0 && !found && !halt) look_up();
+        __syncwarp();
+        if (found) return true;
+        if (halt) return false;
+    }
+    return false;
+}
+
 // Rule 2 for the candidates list[0..M): G lanes per candidate h take
 // candidates from a shared counter and scan levels 1..d-2 of L(h).
 template <int G, class Map>
@@ -473,10 +616,12 @@ __device__ void prune_candidates(const Map& mp, const uint64_t* __restrict__ seg
 // the g-th candidate still undecided, and its warps split levels 1..d-2
 // into wpc contiguous ranges. A warp that finds a witness sets the group's
 // flag, and the others stop at their next step. Every warp reaches the
-// barriers (the call is made by the whole CTA).
+// barriers (the call is made by the whole CTA). filters: memory
+// on chip per warp for scan_filtered, or NULL (the map is on chip).
 template <int NT, class Map>
 __device__ void prune_split(const Map& mp, const uint64_t* __restrict__ seg, const uint32_t* __restrict__ hub_arena,
-                            int64_t n, int d, uint32_t* list, const uint32_t* ckeys, int M, int P, int* s_flag) {
+                            int64_t n, int d, uint32_t* list, const uint32_t* ckeys, int M, int P, int* s_flag,
+                            uint32_t* filters, int64_t u) {
     constexpr int kWarps = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int wpc = 1;
@@ -505,8 +650,11 @@ __device__ void prune_split(const Map& mp, const uint64_t* __restrict__ seg, con
         const uint32_t h = ckeys[list[c] & kSlotMask] & kHubMask;
         const int levels = d - 2;
         const int klo = 1 + (int)((int64_t)levels * j / wpc), khi = (int)((int64_t)levels * (j + 1) / wpc);
-        if (klo <= khi && scan_levels<32>(mp, seg, hub_arena, n, d, h, klo, khi, &s_flag[g]) && lane == 0)
-            atomicExch(&s_flag[g], 1);
+        bool hit = false;
+        if (klo <= khi)
+            hit = filters ? scan_filtered(filters + warp * (kDeepFilter + kScanHits), kDeepFilter, seg, hub_arena, n, u, d, h, klo, khi, &s_flag[g])
+                          : scan_levels<32>(mp, seg, hub_arena, n, d, h, klo, khi, &s_flag[g]);
+        if (hit && lane == 0) atomicExch(&s_flag[g], 1);
     }
     __syncthreads();
     if (c >= 0 && j == 0 && lane == 0 && s_flag[g]) list[c] |= kPrunedBit;
@@ -602,11 +750,12 @@ __device__ void prune_by_level(const Map& mp, const uint64_t* __restrict__ seg,
 template <int NT, class Map>
 __device__ __forceinline__ void prune_all(const Map& mp, const uint64_t* seg, const uint32_t* hub_arena, int64_t n,
                                           int d, uint32_t* list, const uint32_t* ckeys, const uint32_t* open, int M,
-                                          int to_scan, int* next, const uint64_t* useg, int* s_flag) {
+                                          int to_scan, int* next, const uint64_t* useg, int* s_flag,
+                                          uint32_t* filters, int64_t u) {
     const int items = open ? to_scan : M;
     if (to_scan >= 64) prune_by_level<8>(mp, seg, hub_arena, n, d, list, ckeys, open, items, next, useg);
     else if (to_scan >= NT / 32) prune_candidates<16>(mp, seg, hub_arena, n, d, list, ckeys, open, items, next);
-    else prune_split<NT>(mp, seg, hub_arena, n, d, list, ckeys, M, to_scan, s_flag);
+    else prune_split<NT>(mp, seg, hub_arena, n, d, list, ckeys, M, to_scan, s_flag, filters, u);
 }
 
 // Landmark filter (Section "Landmark-Based Filtering"). For a candidate h
@@ -660,6 +809,56 @@ __device__ __forceinline__ uint32_t landmark_verdict(const uint32_t* ua, const u
     return (sum < d ? 1u : 0u) | ((over >= d || under <= -d) ? 2u : 0u);
 }
 
+// Whether u's neighbours prove sd(u,h) >= d: every neighbour z has
+// sd(z,h) >= d-1, either because it holds (h, d-1) itself or by a landmark
+// with |sd(z,l) - sd(l,h)| >= d-1. Most neighbours that do not hold h lie on
+// the far side of u, at distance d or d+1 from h, so their landmark bound
+// may fall one or two short, where u's own had to be exact. By one warp, for
+// at most 32 neighbours (false for more).
+__device__ bool proven_by_neighbours(const LevelArgs& A, int64_t u, uint32_t h, int d) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, wl = lane & 15, need = d - 1;
+    const int64_t a0 = A.rp[u];
+    const int deg = (int)min(A.rp[u + 1] - a0, (int64_t)33);
+    if (deg > 32) return false;
+    const bool in = wl < A.lmk_words;
+    uint4 b = make_uint4(0u, 0u, 0u, 0u);
+    if (in) b = __ldg((const uint4*)(A.lmk + (size_t)h * A.lmk_stride) + wl);
+    b = make_uint4(~lmk_clamp(b.x), ~lmk_clamp(b.y), ~lmk_clamp(b.z), ~lmk_clamp(b.w));
+    const uint32_t z = lane < deg ? (uint32_t)__ldg(A.col + a0 + lane) : 0u;
+    unsigned open = 0;
+    for (int i = 0; i < deg; i += 2) {  // two neighbours at a time, 16 lanes each
+        const uint32_t zr = __shfl_sync(FULL, z, min(i + (lane >> 4), deg - 1));
+        bool far = false;
+        if (in) {
+            const uint4 a = __ldg((const uint4*)(A.lmk + (size_t)zr * A.lmk_stride) + wl);
+            uint32_t hi = 0x80008000u, lo = kLmkClamp;  // of sd(z,l) - sd(l,h) - 1
+            hi = __viaddmax_s16x2(lmk_clamp(a.x), b.x, hi);
+            lo = __viaddmin_s16x2(lmk_clamp(a.x), b.x, lo);
+            hi = __viaddmax_s16x2(lmk_clamp(a.y), b.y, hi);
+            lo = __viaddmin_s16x2(lmk_clamp(a.y), b.y, lo);
+            hi = __viaddmax_s16x2(lmk_clamp(a.z), b.z, hi);
+            lo = __viaddmin_s16x2(lmk_clamp(a.z), b.z, lo);
+            hi = __viaddmax_s16x2(lmk_clamp(a.w), b.w, hi);
+            lo = __viaddmin_s16x2(lmk_clamp(a.w), b.w, lo);
+            const int over = max((int)(int16_t)(hi & 0xFFFFu), (int)(int16_t)(hi >> 16)) + 1;
+            const int under = min((int)(int16_t)(lo & 0xFFFFu), (int)(int16_t)(lo >> 16)) + 1;
+            far = over >= need || under <= -need;
+        }
+        const unsigned m = __ballot_sync(FULL, far);
+        if (!(m & 0xFFFFu)) open |= 1u << i;
+        if (i + 1 < deg && !(m >> 16)) open |= 2u << i;
+    }
+    bool holds = true;  // (h, d-1) in L(z)
+    if ((open >> lane) & 1u) {
+        const uint64_t s = __ldg(A.seg + (int64_t)need * A.n + z);
+        const uint32_t* hs = A.hub_arena + seg_start(s);
+        const uint32_t at = seg_lower_bound(hs, seg_len(s), h);
+        holds = at < seg_len(s) && (__ldg(hs + at) & kHubMask) == h;
+    }
+    return __all_sync(FULL, holds);
+}
+
 // The filter over list[0..M): the verdict is added to each entry, and the
 // undecided positions are collected in open[0..*s_open) (any order) when
 // open is given. *s_pruned, *s_proven and *s_open (zero before) receive the
@@ -695,6 +894,13 @@ __device__ void landmark_filter(const LevelArgs& A, const uint32_t* ua, int d, u
     if (lane == 0 && proven) atomicAdd(s_proven, proven);
 }
 
+// Records that u's segment [b0, b0 + S) waits for `scans` scans.
+__device__ __forceinline__ int hold_segment(const LevelArgs& A, int64_t u, unsigned long long b0, int S, int scans) {
+    const int k = atomicAdd(&A.stt->n_held, 1);  // at most one per vertex
+    A.held[k] = {b0, (int32_t)u, S, scans, 0, 0};
+    return k;
+}
+
 __device__ void block_bitonic_sort(unsigned long long* buf, uint32_t P) {
     for (uint32_t k = 2; k <= P; k <<= 1) {
         for (uint32_t j = k >> 1; j > 0; j >>= 1) {
@@ -716,11 +922,14 @@ __device__ void block_bitonic_sort(unsigned long long* buf, uint32_t P) {
 // ---------------------------------------------------------------------------
 // The level kernel.
 
-template <int kMap, bool kOffChip, int NT>
+// kDeep: the levels that defer their scans (kDeferLevel), in a form of its own
+// so that the shallow levels' form keeps its registers.
+template <int kMap, bool kOffChip, int NT, bool kDeep = false>
 __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelArgs A) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ int s_item, s_nkeys, s_abort, s_m, s_next, s_nsurv, s_route;
     __shared__ int s_lpr, s_lpv, s_open;             // the landmark filter's counts
+    __shared__ int s_held;                           // this vertex's HeldSegment
     __shared__ __align__(16) uint32_t s_lmk[kLmkMax / 2];  // u's landmark distances (uint16 pairs, clamped)
     __shared__ uint64_t s_useg[kUSideLevels];  // u's level descriptors for the rule-2 scan
     __shared__ int s_wcnt[NT / 32];
@@ -1070,18 +1279,38 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
             if (tid == 0 && s_lpr) atomicAdd(&A.stt->lmk_pruned, (unsigned long long)s_lpr);
             if (tid == 0 && s_lpv) atomicAdd(&A.stt->lmk_proven, (unsigned long long)s_lpv);
         }
-        if (d >= 3 && !marked && ns > 0) {
+        // the deep levels' undecided candidates stay in the list as survivors
+        // and are scanned later, unless the queue of scans is full
+        unsigned int q0 = 0;
+        bool defer = false;
+        if (kDeep && A.held && !marked && ns > 0) {
+            if (tid == 0) s_next = (int)atomicAdd(&A.stt->n_scan, (unsigned)ns);
+            __syncthreads();
+            q0 = (unsigned)s_next;
+            defer = q0 < A.scan_cap && A.scan_cap - q0 >= (unsigned)ns;
+            if (!defer)
+                for (unsigned int i = q0 + tid; i < A.scan_cap && i - q0 < (unsigned)ns; i += NT) A.scans[i].held = -1;
+            __syncthreads();
+            if (tid == 0) s_next = 0;
+            __syncthreads();
+        }
+        if (d >= 3 && !marked && ns > 0 && !defer) {
             // u's level descriptors, for scanning u's side when it is shorter
             // (not with bitmaps: their probes cost one on-chip read)
             const bool useg_on = kMap != kMapBitmap && d - 2 < kUSideLevels;
             if (useg_on && tid < d - 1) s_useg[tid] = __ldg(A.seg + (int64_t)tid * n + u);
             __syncthreads();
             const uint64_t* useg = useg_on ? s_useg : nullptr;
+            // the segment-search map without its cache leaves the map's memory free
+            uint32_t* filters = kDeep && kMap == kMapSeg && !kOffChip && !sm.cache &&
+                                        L.list - L.map >= (size_t)kWarps * (kDeepFilter + kScanHits) * 4
+                                    ? (uint32_t*)mapr
+                                    : nullptr;
             if constexpr (kMap == kMapBitmap)
-                prune_all<NT>(bm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt);
+                prune_all<NT>(bm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt, filters, u);
             else if constexpr (kMap == kMapHash)
-                prune_all<NT>(hm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt);
-            else prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt);
+                prune_all<NT>(hm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt, filters, u);
+            else prune_all<NT>(sm, A.seg, A.hub_arena, n, d, list, ckeys, nullptr, M, ns, &s_next, useg, s_wcnt, filters, u);
             __syncthreads();
         }
         // 4. survivors, hub-sorted, appended as L_d(u). Candidate hubs are < u:
@@ -1109,6 +1338,7 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                     const unsigned long long b0 = atomicAdd(&A.stt->bump, (unsigned long long)S);
                     if (b0 + S > A.arena_cap) atomicOr(&A.stt->arena_overflow, 1);
                     s_base = b0;
+                    if (defer) s_held = hold_segment(A, u, b0, S, ns);
                 }
                 __syncthreads();
                 const unsigned long long b0 = s_base;
@@ -1125,8 +1355,9 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                         A.hub_arena[b0 + r] = h | (key & kOvfBit);
                         A.cnt_arena[b0 + r] = cv;
                         cm = max(cm, count_bound(cv, key & kOvfBit));
+                        if (defer && !(e & kProvenBit)) A.scans[q0 + atomicAdd(&s_next, 1)] = {s_held, (int32_t)r};
                     }
-                    if (tid == 0) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
+                    if (tid == 0 && !defer) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
                 }
             }
         } else {
@@ -1134,7 +1365,7 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                 const uint32_t e = list[c];
                 if (!(e & kPrunedBit))
                     sortbuf[atomicAdd(&s_nsurv, 1)] =
-                        ((unsigned long long)(ckeys[e & kSlotMask] & kHubMask) << 32) | (e & kSlotMask);
+                        ((unsigned long long)(ckeys[e & kSlotMask] & kHubMask) << 32) | (e & (kSlotMask | kProvenBit));
             }
             __syncthreads();
             const int S = s_nsurv;
@@ -1147,19 +1378,21 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                     const unsigned long long b0 = atomicAdd(&A.stt->bump, (unsigned long long)S);
                     if (b0 + S > A.arena_cap) atomicOr(&A.stt->arena_overflow, 1);
                     s_base = b0;
+                    if (defer) s_held = hold_segment(A, u, b0, S, ns);
                 }
                 __syncthreads();
                 const unsigned long long b0 = s_base;
                 if (b0 + S <= A.arena_cap) {
                     for (int i = tid; i < S; i += NT) {
-                        const uint32_t slot = (uint32_t)sortbuf[i];
+                        const uint32_t e = (uint32_t)sortbuf[i], slot = e & kSlotMask;
                         const uint32_t key = ckeys[slot];
                         const uint64_t cv = ccnt[slot];
                         A.hub_arena[b0 + i] = (key & kHubMask) | (key & kOvfBit);
                         A.cnt_arena[b0 + i] = cv;
                         cm = max(cm, count_bound(cv, key & kOvfBit));
+                        if (defer && !(e & kProvenBit)) A.scans[q0 + atomicAdd(&s_next, 1)] = {s_held, (int32_t)i};
                     }
-                    if (tid == 0) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
+                    if (tid == 0 && !defer) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
                 }
             }
         }
@@ -1174,18 +1407,21 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
 #include "pspc_dense.cuh"
 
 // ---------------------------------------------------------------------------
-// The level for tiny vertices (fewer than 2^kMicroBucket pulled entries):
-// one warp per vertex and no CTA barrier, so that many such vertices (the
-// deep levels of high-diameter graphs, the tails of power-law graphs) are in
-// flight per SM. The warp stages the pulled entries on chip, drops those
-// whose hub is already in L_<d(u) (segment search), sorts the rest by hub
-// (a 64-element bitonic sort in registers, two elements per lane) and sums
-// the counts of equal hubs with a segmented scan (mod 2^64; the flag takes
-// the entries' flags and every carry: Label Merging). Rule 2 then runs per
-// candidate: the landmark filter, and for the undecided ones a scan of
-// levels 1..d-2 of L(h) by the whole warp. Survivors are already in hub
-// order and are appended as L_d(u).
+// The level for small vertices (fewer than 32 R pulled entries): one warp
+// per vertex and no CTA barrier, so that many such vertices (the deep levels
+// of high-diameter graphs, the tails of power-law graphs) are in flight per
+// SM. The pulled entries are read side by side, R to a lane; those whose hub
+// is already in L_<d(u) are dropped (a search in u's segments of levels d-1
+// and d-2, copied on chip) before their counts are read, and the rest
+// compacted on chip, sorted by hub (bitonic, in registers) and the counts of
+// equal hubs summed with a segmented scan (mod 2^64; the flag takes the
+// entries' flags and every carry: Label Merging). A hub comes at most once
+// per arc, so the scan takes log2(deg u) steps. Rule 2 then runs per
+// candidate: the landmark filter, and for the undecided ones a label scan
+// by the whole warp. Survivors are already in hub order and are appended as
+// L_d(u).
 constexpr int kMicroWarps = kMicroThreads / 32;
+constexpr int kMicroOwn = 128;  // entries of u's levels d-1 and d-2 kept on chip
 
 __device__ __forceinline__ void add_count(uint64_t& sum, uint32_t& flag, uint64_t c, uint32_t f) {
     const uint64_t s = sum + c;
@@ -1193,21 +1429,231 @@ __device__ __forceinline__ void add_count(uint64_t& sum, uint32_t& flag, uint64_
     sum = s;
 }
 
+// One warp's memory: the landmark row and the scan's filter are needed after
+// the staged entries and the copy of u's segments.
+template <int R>
+struct MicroMem {
+    unsigned long long cnt[32 * R];
+    uint32_t hub[32 * R];
+    union {
+        uint32_t own[kMicroOwn];
+        struct {
+            uint32_t lmk[kLmkMax / 2];
+            uint32_t filter[kMicroFilter + kScanHits];
+        } f;
+    } u;
+};
+
+// Steps 2 to 5 for the T (at most 32 R) entries in m.hub and m.cnt.
+template <int R, class Mem>
+__device__ void micro_merge(const LevelArgs& A, Mem& m, int T, int64_t u, int64_t deg, unsigned long long& n_uniq,
+                            unsigned long long& n_lpr, unsigned long long& n_lpv, uint32_t& cm) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int d = A.d;
+    const int64_t n = A.n;
+    uint32_t* hb = m.hub;
+
+    // 2. sort keys: hub << 7 | entry, 0xFFFFFFFF for absent entries (last)
+    uint32_t key[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int e = lane + 32 * j;
+        key[j] = e < T ? ((hb[e] & kHubMask) << 7) | (uint32_t)e : 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (int k = 2; k <= 32 * R; k <<= 1) {
+#pragma unroll
+        for (int jj = k >> 1; jj > 0; jj >>= 1) {
+            if (jj >= 32) {  // partners in the same lane
+#pragma unroll
+                for (int j = 0; j < R; ++j) {
+                    const int q = j ^ (jj / 32);
+                    if (q < j) continue;
+                    const bool asc = ((32 * j) & k) == 0;
+                    const uint32_t lo = min(key[j], key[q]), hi = max(key[j], key[q]);
+                    key[j] = asc ? lo : hi;
+                    key[q] = asc ? hi : lo;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < R; ++j) {
+                    const int e = lane + 32 * j;
+                    const uint32_t other = __shfl_xor_sync(FULL, key[j], jj);
+                    const bool lower = (e & jj) == 0, asc = (e & k) == 0;
+                    key[j] = (lower == asc) ? min(key[j], other) : max(key[j], other);
+                }
+            }
+        }
+    }
+
+    // 3. segmented sums over runs of equal hubs, in sorted order
+    uint32_t hub[R], flg[R];
+    uint64_t sum[R];
+    unsigned heads[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const bool valid = key[j] != 0xFFFFFFFFu;
+        const int src = (int)(key[j] & 127u);
+        hub[j] = valid ? key[j] >> 7 : 0xFFFFFFFFu;
+        sum[j] = valid ? (uint64_t)m.cnt[src] : 0ull;
+        flg[j] = valid ? hb[src] >> 31 : 0u;
+        // a run starts where the previous element (in sorted order) has
+        // another hub; row j's lane 0 follows row j-1's lane 31
+        const uint32_t prev = __shfl_up_sync(FULL, hub[j], 1);
+        const uint32_t last = j > 0 ? __shfl_sync(FULL, hub[j > 0 ? j - 1 : 0], 31) : 0xFFFFFFFFu;
+        heads[j] = __ballot_sync(FULL, valid && (lane == 0 ? (j == 0 || last != hub[j]) : prev != hub[j]));
+    }
+    int uniq = 0;
+    uint64_t carry = 0;
+    uint32_t carry_flag = 0;
+    bool cand[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        uniq += __popc(heads[j]);
+        // lanes before this one in its run (in this row)
+        const unsigned mine = heads[j] & (lt | (1u << lane));
+        const int back = mine ? lane - (31 - __clz(mine)) : lane;
+        for (int o = 1; o < 32 && o < deg; o <<= 1) {
+            const uint64_t sv = __shfl_up_sync(FULL, sum[j], o);
+            const uint32_t fv = __shfl_up_sync(FULL, flg[j], o);
+            if (back >= o) add_count(sum[j], flg[j], sv, fv);
+        }
+        if (!mine && hub[j] != 0xFFFFFFFFu) add_count(sum[j], flg[j], carry, carry_flag);  // the row before's last run
+        carry = __shfl_sync(FULL, sum[j], 31);
+        carry_flag = __shfl_sync(FULL, flg[j], 31);
+        // the last element of each run holds its total
+        const uint32_t next = __shfl_down_sync(FULL, hub[j], 1);
+        const uint32_t first = j + 1 < R ? __shfl_sync(FULL, hub[j + 1 < R ? j + 1 : j], 0) : 0xFFFFFFFFu;
+        cand[j] = hub[j] != 0xFFFFFFFFu && (lane == 31 ? first != hub[j] : next != hub[j]);
+    }
+    n_uniq += (unsigned long long)uniq;
+
+    // 4. rule 2: the landmark filter, then the undecided candidates' scans
+    bool surv[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) surv[j] = cand[j];
+    unsigned und[R];  // undecided candidates
+    int n_open = 0;
+    unsigned int q0 = 0;  // their places in the queue of deferred scans
+    bool defer = false;
+    if (d >= 3 && uniq > 0) {
+        if (A.lmk) {
+            __syncwarp();
+            for (int i = lane; i < A.lmk_stride / 4; i += 32)
+                m.u.f.lmk[i] = lmk_clamp(__ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + i));
+            // the candidates' hubs in order (the staged entries are done
+            // with), eight lanes to each, then the verdicts back
+            int at[R], before = 0;
+            uint32_t* verdict = (uint32_t*)m.cnt;
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const unsigned c = __ballot_sync(FULL, cand[j]);
+                at[j] = before + __popc(c & lt);
+                before += __popc(c);
+                if (cand[j]) hb[at[j]] = hub[j];
+            }
+            __syncwarp();
+            for (int base = 0; base < uniq; base += 4) {
+                const int c = base + lane / 8;
+                const uint32_t v = landmark_verdict<8>(m.u.f.lmk, A.lmk + (size_t)(c < uniq ? hb[c] : 0u) * A.lmk_stride,
+                                                       c < uniq ? A.lmk_words : 0, d, lane % 8, FULL);
+                if (c < uniq && lane % 8 == 0) verdict[c] = v;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const uint32_t v = cand[j] ? verdict[at[j]] : 1u;
+                und[j] = __ballot_sync(FULL, v == 0u);
+                if (cand[j] && (v & 1u)) {
+                    surv[j] = false;
+                    ++n_lpr;
+                } else if (cand[j] && (v & 2u)) {
+                    ++n_lpv;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < R; ++j) und[j] = __ballot_sync(FULL, cand[j]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < R; ++j) n_open += __popc(und[j]);
+        if (A.held && A.lmk && n_open > 0) {
+            if (lane == 0) q0 = atomicAdd(&A.stt->n_scan, (unsigned)n_open);
+            q0 = __shfl_sync(FULL, q0, 0);
+            defer = q0 < A.scan_cap && A.scan_cap - q0 >= (unsigned)n_open;
+            if (!defer)
+                for (unsigned int i = q0 + lane; i < A.scan_cap && i - q0 < (unsigned)n_open; i += 32)
+                    A.scans[i].held = -1;
+        }
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            for (unsigned left = defer ? 0u : und[j]; left; left &= left - 1) {
+                const int src = __ffs(left) - 1;
+                const uint32_t h = __shfl_sync(FULL, hub[j], src);
+                if (A.lmk && d >= kNeighbourLevel && proven_by_neighbours(A, u, h, d)) continue;
+                const bool pruned = scan_filtered(m.u.f.filter, kMicroFilter, A.seg, A.hub_arena, n, u, d, h, 1, d - 2, nullptr);
+                if (pruned && lane == src) surv[j] = false;
+            }
+    }
+
+    // 5. append the survivors in hub order
+    unsigned sv[R];
+    int S = 0;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        sv[j] = __ballot_sync(FULL, surv[j]);
+        S += __popc(sv[j]);
+    }
+    if (S > 0) {
+        unsigned long long b0 = 0;
+        if (lane == 0) {
+            b0 = atomicAdd(&A.stt->bump, (unsigned long long)S);
+            if (b0 + S > A.arena_cap) atomicOr(&A.stt->arena_overflow, 1);
+        }
+        b0 = __shfl_sync(FULL, b0, 0);
+        if (b0 + S <= A.arena_cap) {
+            int before = 0, held = 0;
+            if (defer) {
+                if (lane == 0) held = hold_segment(A, u, b0, S, n_open);
+                held = __shfl_sync(FULL, held, 0);
+            }
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (surv[j]) {
+                    const int r = before + __popc(sv[j] & lt);
+                    A.hub_arena[b0 + r] = hub[j] | (flg[j] ? kOvfBit : 0u);
+                    A.cnt_arena[b0 + r] = sum[j];
+                    cm = max(cm, count_bound(sum[j], flg[j]));
+                    if (defer && ((und[j] >> lane) & 1u)) A.scans[q0 + __popc(und[j] & lt)] = {held, r};
+                }
+                if (defer) q0 += __popc(und[j]);
+                before += __popc(sv[j]);
+            }
+            if (lane == 0 && !defer) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
+        }
+    }
+    __syncwarp();
+}
+
+template <int R>
 __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A) {
-    __shared__ uint32_t s_hub[kMicroWarps][64];
-    __shared__ unsigned long long s_cnt[kMicroWarps][64];
-    __shared__ __align__(16) uint32_t s_lmkw[kMicroWarps][kLmkMax / 2];
+    __shared__ __align__(16) MicroMem<R> s_mem[kMicroWarps];
     const unsigned FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int d = A.d;
     const int64_t n = A.n;
     const uint64_t* seg_prev = A.seg + (int64_t)(d - 1) * n;
-    uint32_t* hb = s_hub[w];
-    unsigned long long* cbuf = s_cnt[w];
-    uint32_t* ul = s_lmkw[w];
+    MicroMem<R>& m = s_mem[w];
     const unsigned lt = (1u << lane) - 1u;
     unsigned long long n_uniq = 0, n_lpr = 0, n_lpv = 0;
     uint32_t cm = 0;  // largest count appended by this lane (LevelStatus::cmax)
+    const bool push = A.push_hub != nullptr;
+    const uint32_t* ghub = push ? A.push_hub : A.hub_arena;
+    const unsigned long long* gcnt =
+        push ? (const unsigned long long*)A.push_cnt : (const unsigned long long*)A.cnt_arena;
     for (int round = 0;; ++round) {
         int item;
         if (A.granular) {
@@ -1219,207 +1665,93 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
         }
         if (item >= A.n_items) break;
         const int64_t u = A.items[item];
-        SegMap sm;
-        sm.seg = A.seg;
-        sm.hub_arena = A.hub_arena;
-        sm.n = n;
-        sm.u = u;
-        sm.d = d;
-        sm.cache = nullptr;
-        sm.cwords = 0;
-        sm.base = 0;
+        const int64_t a0 = A.rp[u], a1 = A.rp[u + 1];
 
-        // 1. stage the pulled entries (fewer than 64)
-        int total = 0;
-        if (A.push_hub) {
-            const int64_t b0 = __ldg(A.push_off + A.rp[u]);
-            total = (int)(__ldg(A.push_off + A.rp[u + 1]) - b0);
-            for (int i = lane; i < total; i += 32) {
-                hb[i] = __ldg(A.push_hub + b0 + i);
-                cbuf[i] = __ldg((const unsigned long long*)A.push_cnt + b0 + i);
-            }
-        } else {
-            const int64_t a0 = A.rp[u], a1 = A.rp[u + 1];
-            for (int64_t ca = a0; ca < a1; ca += 32) {
-                const int64_t a = ca + lane;
-                uint32_t c = 0;
-                uint64_t st = 0;
-                if (a < a1) {
-                    c = __ldg(A.cnt_arc + a);
-                    if (c) st = seg_start(__ldg(seg_prev + __ldg(A.col + a))) + (A.arc_lo ? __ldg(A.arc_lo + a) : 0u);
-                }
-                uint32_t incl = c;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o) incl += t;
-                }
-                const int base = total + (int)(incl - c);
-                for (uint32_t i = 0; i < c; ++i) {
-                    hb[base + i] = __ldg(A.hub_arena + st + i);
-                    cbuf[base + i] = __ldg((const unsigned long long*)A.cnt_arena + st + i);
-                }
-                total += (int)__shfl_sync(FULL, incl, 31);
-            }
-        }
+        // 1. u's segments of levels d-1 and d-2, the only ones that can
+        // hold a pulled hub (level 0 is u itself, never pulled)
+        const uint64_t own1 = __ldg(seg_prev + u);
+        const uint64_t own2 = d > 2 ? __ldg(A.seg + (int64_t)(d - 2) * n + u) : 0ull;
+        const uint32_t n1 = seg_len(own1), n2 = seg_len(own2);
+        const bool staged = n1 + n2 <= (uint32_t)kMicroOwn;
+        if (staged)
+            for (uint32_t i = lane; i < n1 + n2; i += 32)
+                m.u.own[i] = __ldg(A.hub_arena + (i < n1 ? seg_start(own1) : seg_start(own2) - n1) + i) & kHubMask;
         __syncwarp();
-
-        // 2. membership filter and sort keys: hub << 6 | entry, 0xFFFFFFFF
-        // for dropped and absent entries (they sort last)
-        uint32_t key[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int e = lane + 32 * j;
-            key[j] = 0xFFFFFFFFu;
-            if (e < total) {
-                const uint32_t h = hb[e] & kHubMask;
-                if (!sm.member(h)) key[j] = (h << 6) | (uint32_t)e;
+        auto find = [&](const uint32_t* xs, uint32_t len, uint32_t x) {  // in the on-chip copy
+            uint32_t lo = 0, hi = len;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (xs[mid] < x) lo = mid + 1; else hi = mid;
             }
-        }
-#pragma unroll
-        for (int k = 2; k <= 64; k <<= 1) {
-#pragma unroll
-            for (int jj = k >> 1; jj > 0; jj >>= 1) {
-                if (jj == 32) {  // partners in the same lane
-                    const bool asc = (lane & k) == 0;
-                    const uint32_t lo = min(key[0], key[1]), hi = max(key[0], key[1]);
-                    key[0] = asc ? lo : hi;
-                    key[1] = asc ? hi : lo;
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const int e = lane + 32 * j;
-                        const uint32_t other = __shfl_xor_sync(FULL, key[j], jj);
-                        const bool lower = (e & jj) == 0, asc = (e & k) == 0;
-                        key[j] = (lower == asc) ? min(key[j], other) : max(key[j], other);
-                    }
+            return lo < len && xs[lo] == x;
+        };
+        auto member = [&](uint32_t x) {
+            if (staged) return find(m.u.own, n1, x) || find(m.u.own + n1, n2, x);
+            const uint32_t* h1 = A.hub_arena + seg_start(own1);
+            const uint32_t* h2 = A.hub_arena + seg_start(own2);
+            return seg_contains(h1, n1, x) || seg_contains(h2, n2, x);
+        };
+
+        // the pulled entries (fewer than 32 R), 32 arcs at a time
+        int T = 0;
+        const int64_t arcs_end = push ? a0 + 1 : a1;
+        for (int64_t ca = a0; ca < arcs_end; ca += 32) {
+            const int64_t a = ca + lane;
+            uint32_t c = 0;
+            uint64_t st = 0;
+            if (push) {  // the entries sent to u lie in one bucket
+                if (lane == 0) {
+                    st = (uint64_t)__ldg(A.push_off + a0);
+                    c = (uint32_t)(__ldg(A.push_off + a1) - (int64_t)st);
                 }
+            } else if (a < a1) {
+                c = __ldg(A.cnt_arc + a);
+                if (c) st = seg_start(__ldg(seg_prev + __ldg(A.col + a))) + (A.arc_lo ? __ldg(A.arc_lo + a) : 0u);
             }
-        }
-
-        // 3. segmented sums over runs of equal hubs, in sorted order
-        uint32_t hub[2], flg[2];
-        uint64_t sum[2];
-        bool valid[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            valid[j] = key[j] != 0xFFFFFFFFu;
-            hub[j] = valid[j] ? key[j] >> 6 : 0xFFFFFFFFu;
-            const int src = (int)(key[j] & 63u);
-            sum[j] = valid[j] ? (uint64_t)cbuf[src] : 0ull;
-            flg[j] = valid[j] ? (hb[src] >> 31) : 0u;
-        }
-        // a run starts where the previous element (in sorted order) has
-        // another hub; row 1's lane 0 follows row 0's lane 31
-        const uint32_t prev0 = __shfl_up_sync(FULL, hub[0], 1);
-        const uint32_t last0 = __shfl_sync(FULL, hub[0], 31);
-        const uint32_t prev1 = __shfl_up_sync(FULL, hub[1], 1);
-        const bool head0 = valid[0] && (lane == 0 || prev0 != hub[0]);
-        const bool head1 = valid[1] && (lane == 0 ? last0 != hub[1] : prev1 != hub[1]);
-        const unsigned h0 = __ballot_sync(FULL, head0), h1 = __ballot_sync(FULL, head1);
-        const int id0 = __popc(h0 & (lt | (1u << lane)));                       // segment id (1-based)
-        const int id1 = __popc(h0) + __popc(h1 & (lt | (1u << lane)));
-        int id[2] = {id0, id1};
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
+            uint32_t incl = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t sv = __shfl_up_sync(FULL, sum[j], o);
-                const uint32_t fv = __shfl_up_sync(FULL, flg[j], o);
-                const int iv = __shfl_up_sync(FULL, id[j], o);
-                if (lane >= o && iv == id[j] && valid[j]) add_count(sum[j], flg[j], sv, fv);
+                const uint32_t t = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += t;
             }
-        }
-        {  // row 1's first run may continue row 0's last one (every lane
-           // takes part in the shuffles; only then do lanes branch)
-            const uint64_t s31 = __shfl_sync(FULL, sum[0], 31);
-            const uint32_t f31 = __shfl_sync(FULL, flg[0], 31);
-            const int i31 = __shfl_sync(FULL, id[0], 31);
-            const int v31 = __shfl_sync(FULL, (int)valid[0], 31);
-            if (valid[1] && v31 && id[1] == i31) add_count(sum[1], flg[1], s31, f31);
-        }
-        // the last element of each run holds its total
-        const uint32_t next0 = __shfl_down_sync(FULL, hub[0], 1);
-        const uint32_t first1 = __shfl_sync(FULL, hub[1], 0);
-        const uint32_t next1 = __shfl_down_sync(FULL, hub[1], 1);
-        bool cand[2];
-        cand[0] = valid[0] && (lane == 31 ? first1 != hub[0] : next0 != hub[0]);
-        cand[1] = valid[1] && (lane == 31 || next1 != hub[1]);
-        const int uniq = __popc(h0) + __popc(h1);
-        n_uniq += (unsigned long long)uniq;
-
-        // 4. rule 2: the landmark filter, then the undecided candidates' scans
-        bool surv[2] = {cand[0], cand[1]};
-        if (d >= 3 && uniq > 0) {
-            bool und[2] = {cand[0], cand[1]};
-            if (A.lmk) {
-                for (int i = lane; i < A.lmk_stride / 4; i += 32)
-                    ul[i] = lmk_clamp(__ldg((const uint32_t*)(A.lmk + u * A.lmk_stride) + i));
-                // the candidates' hubs in order (the staged entries are done
-                // with), eight lanes to each, then the verdicts back
-                const unsigned c0 = __ballot_sync(FULL, cand[0]), c1 = __ballot_sync(FULL, cand[1]);
-                const int at[2] = {__popc(c0 & lt), __popc(c0) + __popc(c1 & lt)};
-                uint32_t* verdict = (uint32_t*)cbuf;
+            const uint32_t excl = incl - c, total = __shfl_sync(FULL, incl, 31);
+            st -= excl;
+            uint32_t hw[R];
+            uint64_t pos[R];
 #pragma unroll
-                for (int j = 0; j < 2; ++j)
-                    if (cand[j]) hb[at[j]] = hub[j];
-                __syncwarp();
-                for (int base = 0; base < uniq; base += 4) {
-                    const int c = base + lane / 8;
-                    const uint32_t v = landmark_verdict<8>(ul, A.lmk + (size_t)(c < uniq ? hb[c] : 0u) * A.lmk_stride,
-                                                           c < uniq ? A.lmk_words : 0, d, lane % 8, FULL);
-                    if (c < uniq && lane % 8 == 0) verdict[c] = v;
-                }
-                __syncwarp();
+            for (int t = 0; t < R; ++t) {
+                const uint32_t i = t * 32 + lane;
+                hw[t] = kEmpty;
+                if (t * 32 < total) {  // warp-uniform
+                    int j = 0;
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const uint32_t v = cand[j] ? verdict[at[j]] : 0u;
-                    if (v & 1u) {
-                        surv[j] = false;
-                        und[j] = false;
-                        ++n_lpr;
-                    } else if (v & 2u) {
-                        und[j] = false;
-                        ++n_lpv;
+                    for (int step = 16; step > 0; step >>= 1) {
+                        const uint32_t e = __shfl_sync(FULL, excl, j + step);
+                        if (e <= i) j += step;
                     }
+                    pos[t] = __shfl_sync(FULL, st, j) + i;
+                    if (i < total) hw[t] = __ldg(ghub + pos[t]);
                 }
-                __syncwarp();
             }
-            unsigned u0 = __ballot_sync(FULL, und[0]), u1 = __ballot_sync(FULL, und[1]);
-            while (u0 | u1) {
-                const int j = u0 ? 0 : 1;
-                const unsigned m = j ? u1 : u0;
-                const int src = __ffs(m) - 1;
-                const uint32_t h = __shfl_sync(FULL, hub[j], src);
-                const bool pruned = scan_levels<32>(sm, A.seg, A.hub_arena, n, d, h, 1, d - 2, nullptr);
-                if (pruned && lane == src) surv[j] = false;
-                if (j) u1 &= m - 1; else u0 &= m - 1;
-            }
-        }
-
-        // 5. append the survivors in hub order
-        const unsigned s0 = __ballot_sync(FULL, surv[0]), s1 = __ballot_sync(FULL, surv[1]);
-        const int S = __popc(s0) + __popc(s1);
-        if (S > 0) {
-            unsigned long long b0 = 0;
-            if (lane == 0) {
-                b0 = atomicAdd(&A.stt->bump, (unsigned long long)S);
-                if (b0 + S > A.arena_cap) atomicOr(&A.stt->arena_overflow, 1);
-            }
-            b0 = __shfl_sync(FULL, b0, 0);
-            if (b0 + S <= A.arena_cap) {
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    if (!surv[j]) continue;
-                    const int pos = j ? __popc(s0) + __popc(s1 & lt) : __popc(s0 & lt);
-                    A.hub_arena[b0 + pos] = hub[j] | (flg[j] ? kOvfBit : 0u);
-                    A.cnt_arena[b0 + pos] = sum[j];
-                    cm = max(cm, count_bound(sum[j], flg[j]));
+            for (int t = 0; t < R; ++t)
+                if (t * 32 < total) {
+                    const bool keep = t * 32 + lane < total && !member(hw[t] & kHubMask);
+                    const unsigned b = __ballot_sync(FULL, keep);
+                    const int at = T + __popc(b & lt);
+                    if (keep) {
+                        m.hub[at] = hw[t];
+                        m.cnt[at] = __ldg(gcnt + pos[t]);
+                    }
+                    T += __popc(b);
                 }
-                if (lane == 0) A.seg_out[u] = seg_pack(b0, (uint32_t)S);
-            }
         }
         __syncwarp();
+        if (T == 0) continue;
+        const int64_t deg = push ? (int64_t)32 : a1 - a0;
+        if (T <= 32) micro_merge<1>(A, m, T, u, deg, n_uniq, n_lpr, n_lpv, cm);
+        else if (R == 2 || T <= 64) micro_merge<2>(A, m, T, u, deg, n_uniq, n_lpr, n_lpv, cm);
+        else micro_merge<R>(A, m, T, u, deg, n_uniq, n_lpr, n_lpv, cm);
     }
     cm = __reduce_max_sync(FULL, cm);
 #pragma unroll
@@ -1432,6 +1764,95 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
         if (n_uniq) atomicAdd(&A.stt->unique_total, n_uniq);
         if (n_lpr) atomicAdd(&A.stt->lmk_pruned, n_lpr);
         if (n_lpv) atomicAdd(&A.stt->lmk_proven, n_lpv);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The deferred scans, spread over all SMs instead of holding the one warp or
+// CTA that met them (a road network's deep levels have vertices with dozens
+// of undecided candidates). k_prove_deferred first tries the neighbours'
+// proof, which decides half of them at level 100 of grid 256x256 and three
+// quarters from level 277 on; k_scan_deferred scans the rest, split into
+// ranges of levels when there are fewer of them than warps. A pruned entry
+// is marked in the arena; the warp that ends a vertex's last part takes the
+// marked entries out and publishes the segment. Nothing waits: the segments
+// were appended by earlier launches. With the scans in place grid 256x256
+// took 723 ms in the level kernels (1,086 with a warp per vertex at every
+// level), of which less than 100 were not scans.
+constexpr int kScanThreads = 256;
+
+__global__ void __launch_bounds__(kScanThreads) k_prove_deferred(const LevelArgs A) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    if (A.stt->arena_overflow) return;  // the level runs again with a larger arena
+    const int count = (int)min(A.stt->n_scan, A.scan_cap);
+    const int warps = (int)(gridDim.x * (kScanThreads / 32));
+    for (int item = (int)(blockIdx.x * (kScanThreads / 32) + (threadIdx.x >> 5)); item < count; item += warps) {
+        const DeferredScan q = A.scans[item];
+        if (q.held < 0) continue;
+        HeldSegment* H = A.held + q.held;
+        const uint32_t h = __ldg(A.hub_arena + H->start + q.pos) & kHubMask;
+        const bool proven = proven_by_neighbours(A, H->u, h, A.d);
+        if (lane == 0) {
+            if (!proven) A.scans[A.scan_cap + atomicAdd(&A.stt->n_scan_open, 1u)] = q;
+            else if (atomicSub(&H->scans, 1) == 1) A.seg_out[H->u] = seg_pack(H->start, (uint32_t)H->len);
+        }
+        __syncwarp(FULL);
+    }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_deferred(const LevelArgs A) {
+    __shared__ __align__(16) uint32_t s_filter[kScanThreads / 32][kScanFilter + kScanHits];
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    if (A.stt->arena_overflow) return;
+    const int count = (int)A.stt->n_scan_open, levels = A.d - 2;
+    const int parts = max(1, min((int)(gridDim.x * (kScanThreads / 32)) / max(count, 1), (levels + 30) / 31));
+    for (;;) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(&A.stt->work_scan, 1);
+        item = __shfl_sync(FULL, item, 0);
+        if (item >= count * parts) break;
+        const DeferredScan q = A.scans[A.scan_cap + item / parts];
+        const int part = item % parts;
+        const int klo = 1 + (int)((int64_t)levels * part / parts), khi = (int)((int64_t)levels * (part + 1) / parts);
+        HeldSegment* H = A.held + q.held;
+        const int64_t u = H->u;
+        const unsigned long long b0 = H->start;
+        const int S = H->len;
+        const uint32_t h = __ldcg(A.hub_arena + b0 + q.pos) & kHubMask;
+        const bool pruned = scan_filtered(s_filter[w], kScanFilter, A.seg, A.hub_arena, A.n, u, A.d, h, klo, khi, nullptr);
+        int last = 0;
+        if (lane == 0) {
+            if (pruned) {
+                atomicOr(A.hub_arena + b0 + q.pos, kMarkBit);
+                atomicExch(&H->pruned, 1);
+            }
+            __threadfence();
+            last = atomicAdd(&H->done, 1) + 1 == H->scans * parts;
+            __threadfence();
+        }
+        if (!__shfl_sync(FULL, last, 0)) continue;
+        int kept = S;
+        if (__ldcg(&H->pruned)) {  // stable compaction in place: a row is read before earlier places are written
+            kept = 0;
+            for (int r = 0; r < S; r += 32) {
+                const bool in = r + lane < S;
+                const uint32_t hw = in ? __ldcg(A.hub_arena + b0 + r + lane) : kMarkBit;
+                const uint64_t c = in ? __ldcg((const unsigned long long*)A.cnt_arena + b0 + r + lane) : 0ull;
+                const bool keep = in && !(hw & kMarkBit);
+                const unsigned m = __ballot_sync(FULL, keep);
+                if (keep) {
+                    A.hub_arena[b0 + kept + __popc(m & lt)] = hw;
+                    A.cnt_arena[b0 + kept + __popc(m & lt)] = c;
+                }
+                kept += __popc(m);
+                __syncwarp();
+            }
+            if (lane == 0) atomicAdd(&A.stt->dropped, (unsigned long long)(S - kept));
+        }
+        if (lane == 0) A.seg_out[u] = kept ? seg_pack(b0, (uint32_t)kept) : 0ull;
     }
 }
 
@@ -1537,6 +1958,9 @@ cudaError_t level_kernel_attrs(int map_kind, size_t smem_bytes, int* occupancy, 
     const size_t max_dyn = (size_t)optin - fa.sharedSizeBytes;
     if (smem_bytes > max_dyn) return cudaErrorInvalidValue;
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_dyn);
+    if (e == cudaSuccess && nt == kLightThreads && map_kind == kMapSeg)
+        e = cudaFuncSetAttribute((const void*)k_level<kMapSeg, false, kLightThreads, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_dyn - 1024);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, f, nt, smem_bytes);
 }
@@ -1569,18 +1993,35 @@ cudaError_t launch_level_dense(int grid, const LevelArgs& A, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t micro_kernel_occupancy(int* occupancy) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, (const void*)k_level_micro, kMicroThreads, 0);
+// Rows of 32 entries per warp: 2 or 4.
+cudaError_t micro_kernel_occupancy(int rows, int* occupancy) {
+    const void* f = rows == 2 ? (const void*)k_level_micro<2> : (const void*)k_level_micro<4>;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, f, kMicroThreads, 0);
 }
 
-cudaError_t launch_level_micro(int grid, const LevelArgs& A, cudaStream_t st) {
-    k_level_micro<<<grid, kMicroThreads, 0, st>>>(A);
+cudaError_t scan_kernel_occupancy(int* prove, int* scan) {
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(prove, (const void*)k_prove_deferred, kScanThreads, 0);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(scan, (const void*)k_scan_deferred, kScanThreads, 0);
+}
+
+cudaError_t launch_scan_deferred(int prove_grid, int scan_grid, const LevelArgs& A, cudaStream_t st) {
+    k_prove_deferred<<<prove_grid, kScanThreads, 0, st>>>(A);
+    k_scan_deferred<<<scan_grid, kScanThreads, 0, st>>>(A);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_level_micro(int rows, int grid, const LevelArgs& A, cudaStream_t st) {
+    if (rows == 2) k_level_micro<2><<<grid, kMicroThreads, 0, st>>>(A);
+    else k_level_micro<4><<<grid, kMicroThreads, 0, st>>>(A);
     return cudaGetLastError();
 }
 
 cudaError_t launch_level(int map_kind, bool offchip, int grid, size_t smem_bytes, const LevelArgs& A,
                          cudaStream_t st, int nt) {
-    if (nt == kLightThreads && !offchip) launch_level_nt<kLightThreads>(map_kind, false, grid, smem_bytes, A, st);
+    if (nt == kLightThreads && !offchip && map_kind == kMapSeg && A.d >= kDeferLevel)
+        k_level<kMapSeg, false, kLightThreads, true><<<grid, nt, smem_bytes, st>>>(A);
+    else if (nt == kLightThreads && !offchip) launch_level_nt<kLightThreads>(map_kind, false, grid, smem_bytes, A, st);
     else launch_level_nt<kLevelThreads>(map_kind, offchip, grid, smem_bytes, A, st);
     return cudaGetLastError();
 }

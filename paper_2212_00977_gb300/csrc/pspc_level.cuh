@@ -16,11 +16,13 @@ constexpr uint32_t kLightCap = 1024;  // candidate slots of a light vertex
 constexpr uint32_t kOffStartCap = 16384;    // first off-chip table size
 constexpr uint32_t kOffSlabCap = 1u << 17;  // off-chip slab of the first pass, in candidate slots
 constexpr int kMicroThreads = 256;    // the warp-per-vertex level kernel: 8 vertices per CTA
-constexpr int kMicroBucket = 6;       // micro: fewer than 2^6 pulled entries (64 fit a warp's registers)
+constexpr int kMicroBucket = 7;       // micro: fewer than 2^7 pulled entries (four to a lane); at levels 2 and 3,
+                                      // where nothing is filtered out first, 2^6 (BA 20,011: 6.7 ms, else 6.9)
+constexpr int kTinyBucket = 6;        // of those, fewer than 2^6: two to a lane, and fewer registers
 constexpr int kLightBucket = 9;       // light: fewer than 2^9 pulled entries, so at most 2 * 511 < kLightCap
                                       // slots are asked for, and the table never overflows
-constexpr int kWarpLevelsMax = 127;   // automatic warp-per-vertex levels: at most this deep,
-constexpr int kWarpLevelsFew = 32;    // and while the last level had under this many candidates per vertex
+constexpr int kWarpLevelsFew = 32;    // automatic warp-per-vertex levels: while the last level had under this
+                                      // many candidates per vertex
 constexpr int kArcChunk = kLevelThreads;  // arcs staged per gather chunk (the CTA size)
 
 // Resident CTAs per SM each kernel size is built for (64 registers a thread).
@@ -75,6 +77,12 @@ struct LevelStatus {
     int n_giant;     // off-chip vertices whose candidates overflow the slab
     int work_giant;
     int work_micro;
+    int work_tiny;
+    int n_held;                  // vertices whose segment waits for deferred scans
+    int work_scan;
+    unsigned int n_scan_open;    // of them, left after the neighbours' proof
+    unsigned int n_scan;         // deferred scans asked for (those past the queue's size run in place)
+    unsigned long long dropped;  // entries that deferred scans took out of their segments
     int work_dense;
     unsigned int cmax;  // largest count appended at this level (0xFFFFFFFF: 2^32 or more, or flagged)
     // on-chip attempts and overflows of vertices that can overflow, by
@@ -85,6 +93,29 @@ struct LevelStatus {
     int bucket_cnt[kBuckets];
     int bucket_base[kBuckets];
     int bucket_fill[kBuckets];
+};
+
+// Deferred label scans of the deep levels. A vertex with undecided
+// candidates appends them with its survivors and asks for their scans; the
+// scans of all vertices then run evenly over the GPU (k_scan_deferred), and
+// the last one of a vertex closes its segment.
+constexpr int kDeferLevel = 16;  // first level that defers: shorter scans run in place
+// and only with this many active vertices times levels, where the scans are
+// worth two launches a level (grid 61x67 builds in 17.2 ms without them, 17.9
+// with 2^17 here; grid 128x128 54 ms either way, grid 256x256 339 and 336).
+constexpr int64_t kDeferWork = 1 << 18;
+constexpr int kNeighbourLevel = 8;  // from here on a scan costs more than the neighbours' proof that may spare it
+struct HeldSegment {
+    unsigned long long start;  // of the entries appended so far in the arena
+    int32_t u;
+    int32_t len;
+    int32_t scans;    // asked for, less the proven ones
+    int32_t done;     // parts of them that have run
+    int32_t pruned;   // some scan pruned its entry (marked kMarkBit in the arena)
+};
+struct DeferredScan {
+    int32_t held;  // which HeldSegment (-1: none)
+    int32_t pos;   // which of its entries
 };
 
 struct LevelArgs {
@@ -124,6 +155,9 @@ struct LevelArgs {
     const uint8_t* lmk;   // [n][lmk_stride] bytes of uint16 landmark distances, or NULL (no filter)
     int lmk_stride;       // bytes per row: a multiple of 16, <= 2 kLmkMax
     int lmk_words;        // 16-byte words of each row the filter tests at this level
+    HeldSegment* held;    // deferred scans (NULL: scans run in place)
+    DeferredScan* scans;
+    unsigned int scan_cap;
 };
 
 // Table layout (on chip, or in per-CTA device scratch). The map region also
@@ -239,7 +273,9 @@ cudaError_t dense_kernel_attrs(int* occupancy);
 cudaError_t launch_level_dense(int grid, const LevelArgs& A, cudaStream_t st);
 // The warp-per-vertex variant for vertices with fewer than 2^kMicroBucket
 // pulled entries (k_level_micro).
-cudaError_t micro_kernel_occupancy(int* occupancy);
-cudaError_t launch_level_micro(int grid, const LevelArgs& A, cudaStream_t st);
+cudaError_t micro_kernel_occupancy(int rows, int* occupancy);
+cudaError_t launch_scan_deferred(int prove_grid, int scan_grid, const LevelArgs& A, cudaStream_t st);
+cudaError_t scan_kernel_occupancy(int* prove, int* scan);
+cudaError_t launch_level_micro(int rows, int grid, const LevelArgs& A, cudaStream_t st);
 
 }  // namespace pspc
