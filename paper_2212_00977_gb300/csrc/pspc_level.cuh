@@ -91,7 +91,6 @@ struct LevelStatus {
     unsigned int route_att[kBuckets];
     unsigned int route_ovf[kBuckets];
     int bucket_cnt[kBuckets];
-    int bucket_base[kBuckets];
     int bucket_fill[kBuckets];
 };
 
