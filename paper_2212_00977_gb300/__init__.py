@@ -266,7 +266,7 @@ class Index:
 
     def set_query_group(self, lanes: int) -> None:
         """Query variant of pspc_query: 8/16/32 lanes per pair, 64/128/256
-        staged chunk entries, PSPC_QUERY_BY_SOURCE (L(s) on chip for the
+        a warp per pair through shared memory, PSPC_QUERY_BY_SOURCE (L(s) on chip for the
         pairs of each source: a position table when it fits, else a hash),
         PSPC_QUERY_BY_SOURCE_HASH (the hash form), or 0 = automatic."""
         rc = load().pspc_set_query_group(self._h, int(lanes))

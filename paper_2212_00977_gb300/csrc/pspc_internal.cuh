@@ -47,7 +47,13 @@ struct Index {
     int32_t* rank = nullptr;   // caller id -> rank id
     int32_t* order = nullptr;  // rank id -> caller id
     int64_t* off = nullptr;    // [n+1]
-    int32_t* hub = nullptr;    // hub rank ids
+    // Words: hub rank id << sh | distance << cb | count, with all ones in the
+    // count's cb bits for a count that they cannot hold or that is flagged.
+    // sh = db + cb is at most 16; all three are 0 (a word is the hub alone)
+    // where hub and distance do not fit one word.
+    int32_t* hub = nullptr;
+    int sh = 0, db = 0, cb = 0;
+    int64_t escapes = 0;       // entries whose count is not in their word
     uint16_t* dist = nullptr;  // distance | overflow << 15
     uint64_t* cnt = nullptr;   // trough path count mod 2^64
     int64_t entries = 0;

@@ -4,16 +4,17 @@
 // (Section "Reduction by Equivalence Relation", parallel query evaluation).
 //
 // Kernels: k_query<G> (G lanes per pair, 32-bit hub words in registers,
-// binary search by shuffles), k_query_chunked<CH> (a warp per pair, chunks
-// of CH entries of both labels staged in shared memory, binary search per
-// entry; the side whose last hub is smaller advances), k_query_by_source
-// (pairs sorted by source; L(s) hashed on chip once per run of pairs with
-// that source, each warp streams L(t)). In each, a match h gives
-// dist_s(h) + dist_t(h); counts (and their 128-bit product) are read only
-// for matches that reach the lane's running minimum. The warp then keeps
-// the global minimum and adds the products of the hubs that reach it,
-// modulo 2^64, with a sticky overflow flag (flag of a factor, high word of
-// a product, carry of a sum).
+// binary search by shuffles), k_query_words and k_query_words_split (an index
+// whose entries fit 32-bit words: a hash of one label on chip, the other's
+// words stream past it), k_query_chunked<CH> (a warp per pair, chunks of CH
+// entries of both labels staged in shared memory, binary search per entry;
+// the side whose last hub is smaller advances), k_query_by_source and
+// k_query_by_source_direct (pairs sorted by source; L(s) on chip once per run
+// of pairs with that source, each warp streams L(t)). In each, a match h gives
+// dist_s(h) + dist_t(h), and counts (with their 128-bit product) matter only
+// at the running minimum. The warp then keeps the global minimum and adds the
+// products of the hubs that reach it, modulo 2^64, with a sticky overflow flag
+// (flag of a factor, high word of a product, carry of a sum).
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -37,7 +38,8 @@ struct QueryArgs {
     int64_t n;
     const int32_t* rank;
     const int64_t* off;
-    const int32_t* hub;
+    const int32_t* hub;  // words (Index::hub)
+    int sh, cb, db;      // their layout
     const uint16_t* dist;
     const uint64_t* cnt;
     const int32_t* pairs;
@@ -128,8 +130,8 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(const QueryArgs Q) {
         uint32_t flag = 0;
         while (ia < ea && ib < eb) {
             const bool va = ia + lane < ea, vb = ib + lane < eb;
-            const uint32_t ha = va ? (uint32_t)__ldg(Q.hub + ia + lane) : kNoHub;
-            const uint32_t hb = vb ? (uint32_t)__ldg(Q.hub + ib + lane) : kNoHub;
+            const uint32_t ha = va ? (uint32_t)__ldg(Q.hub + ia + lane) >> Q.sh : kNoHub;
+            const uint32_t hb = vb ? (uint32_t)__ldg(Q.hub + ib + lane) >> Q.sh : kNoHub;
             const uint16_t db = vb ? __ldg(Q.dist + ib + lane) : 0;
             const int la = ea - ia > G ? G - 1 : (int)(ea - ia - 1);
             const int lb = eb - ib > G ? G - 1 : (int)(eb - ib - 1);
@@ -192,11 +194,347 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(const QueryArgs Q) {
     }
 }
 
-// Warp per pair over chunks of CH entries staged in the warp's slice of
-// shared memory (one load round trip per chunk instead of one per 32
-// entries). Each lane looks up its A hubs in the B chunk by binary search;
-// the side whose last hub is smaller advances, and only that side is
-// reloaded.
+// One label looked up in another: lane i searches for entry i of [a, ea) in
+// [b, eb). An isolated vertex's label is one entry whose hub ranks below
+// most others, and merging it reads all of the other label (half of the
+// uniform pairs of an R-MAT graph have one).
+// Each entry costs a search of some fourteen dependent loads, so the other
+// label has to be so many times longer.
+__device__ __forceinline__ bool is_brief(int64_t len, int64_t other) {
+    return len <= 64 ? len * 8 <= other : len <= 512 && len * 16 <= other;
+}
+
+__device__ __forceinline__ void look_up_label(const QueryArgs& Q, int64_t a, int64_t ea, int64_t b, int64_t eb, int lane,
+                                           uint32_t& best, uint64_t& sum, uint32_t& flag) {
+    for (int64_t i = a + lane; i < ea; i += 32) {
+        const uint32_t h = (uint32_t)__ldg(Q.hub + i) >> Q.sh;
+        int64_t lo = b, hi = eb;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (((uint32_t)__ldg(Q.hub + mid) >> Q.sh) < h) lo = mid + 1; else hi = mid;
+        }
+        if (lo == eb || (uint32_t)__ldg(Q.hub + lo) >> Q.sh != h) continue;
+        const uint32_t da = __ldg(Q.dist + i), d2 = __ldg(Q.dist + lo);
+        const uint32_t dsum = (da & 0x7FFFu) + (d2 & 0x7FFFu);
+        if (dsum > best) continue;
+        const uint64_t ca = __ldg((const unsigned long long*)Q.cnt + i);
+        const uint64_t cb = __ldg((const unsigned long long*)Q.cnt + lo);
+        const uint32_t tf = ((da | d2) >> 15) | (uint32_t)(__umul64hi(ca, cb) != 0);
+        if (dsum < best) {
+            best = dsum;
+            sum = ca * cb;
+            flag = tf;
+        } else {
+            add_term(sum, flag, ca * cb, tf);
+        }
+    }
+}
+
+// The query on words (Index::hub): 4 bytes an entry hold hub, distance and a
+// small count, so most pairs read nothing else. (With hub and distance in 6
+// bytes, and the counts of each match at a lane's minimum in sectors of 32
+// bytes, the counts were most of the traffic: 7.5 KB of DRAM reads a pair on
+// R-MAT 65,536.)
+//
+// A warp takes `per` pairs, neighbours in the source order where the call
+// sorted them, reads where all their labels lie at once (a lane each), and
+// joins them source by source: kWordSegment entries of L(s) at a time go into
+// a hash in the warp's slice of shared memory, buckets of four words that one
+// 16-byte read returns, and the part of every L(t) up to the segment's last
+// hub streams past it. No barrier but the warp's own, and no search: the
+// staged merge-join it replaces spent eight dependent on-chip reads on each
+// entry of L(s) and 3,530 instructions on a pair of R-MAT 65,536 (a CTA per
+// source with a table over every hub needs 1,480, but waits at barriers for
+// twice as long as it runs).
+constexpr int kWordBuckets = 256;        // per warp: 4 KB, so that five CTAs share an SM
+constexpr uint32_t kWordSegment = 384;   // entries of L(s) in the hash: 1.5 a bucket
+constexpr int kWordUnroll = 4;           // rows of L(t) in flight
+constexpr size_t kWordBytes = (size_t)(kQueryThreads / 32) * kWordBuckets * 16;
+
+__device__ __forceinline__ uint32_t word_bucket(uint32_t h) { return h * 0x9E3779B1u >> 24; }
+
+// L(s) entries [i0, i1) (words at A) into the warp's hash.
+__device__ __forceinline__ void fill_words(uint32_t* tab, const int32_t* __restrict__ A, uint32_t i0, uint32_t i1,
+                                           int sh, int lane) {
+    for (int i = lane; i < kWordBuckets; i += 32) ((uint4*)tab)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    __syncwarp();
+    for (uint32_t i = i0 + lane; i < i1; i += 32) {
+        const uint32_t w = (uint32_t)__ldg(A + i);
+        uint32_t at = word_bucket(w >> sh) * 4;
+        while (atomicCAS(&tab[at], kNoHub, w) != kNoHub) at = (at + 1) & (kWordBuckets * 4 - 1);
+    }
+    __syncwarp();
+}
+
+// Entries [j, je) of L(t) (words at B, entry 0 at position b0) against the
+// hash of L(s) entries [i0, i1) (entry 0 at a0), as far as hub hi; lanes keep
+// their own minimum and sum. Returns the first entry whose hub is above hi.
+__device__ __forceinline__ uint32_t probe_words(const QueryArgs& Q, const uint32_t* tab, int64_t a0, uint32_t i0,
+                                                uint32_t i1, int64_t b0, uint32_t j, uint32_t je, uint32_t hi, int lane,
+                                                uint32_t& best, uint64_t& sum, uint32_t& flag) {
+    const uint32_t low = (1u << Q.sh) - 1u, dmask = (1u << Q.db) - 1u, cmask = (1u << Q.cb) - 1u;
+    const uint32_t end = hi << Q.sh | low;
+    const int32_t* B = Q.hub + b0;
+    for (; j < je; j += 32 * kWordUnroll) {
+        uint32_t w[kWordUnroll];
+#pragma unroll
+        for (int k = 0; k < kWordUnroll; ++k) w[k] = j + 32 * k + lane < je ? (uint32_t)__ldg(B + j + 32 * k + lane) : kNoHub;
+#pragma unroll
+        for (int k = 0; k < kWordUnroll; ++k) {
+            if (w[k] > end || w[k] == kNoHub) continue;  // (hi can be the largest hub that a word holds)
+            uint32_t b = word_bucket(w[k] >> Q.sh);
+            uint32_t e = kNoHub;  // the word of L(s) with this hub
+            for (;;) {
+                const uint4 v = ((const uint4*)tab)[b];
+                e = (v.x ^ w[k]) <= low ? v.x : (v.y ^ w[k]) <= low ? v.y : (v.z ^ w[k]) <= low ? v.z
+                                                                       : (v.w ^ w[k]) <= low ? v.w : kNoHub;
+                if (e != kNoHub || v.w == kNoHub) break;
+                b = (b + 1) & (kWordBuckets - 1);
+            }
+            const uint32_t dsum = (e >> Q.cb & dmask) + (w[k] >> Q.cb & dmask);
+            if (e == kNoHub || dsum > best) continue;
+            uint64_t ca = e & cmask, cb = w[k] & cmask;
+            uint32_t tf = 0;
+            if (ca == cmask || cb == cmask) {  // a count that a word cannot hold
+                uint32_t lo = i0, up = i1;
+                while (lo < up) {
+                    const uint32_t mid = (lo + up) >> 1;
+                    if ((uint32_t)__ldg(Q.hub + a0 + mid) < e) lo = mid + 1; else up = mid;
+                }
+                const int64_t jj = b0 + j + 32 * k + lane;
+                ca = __ldg((const unsigned long long*)Q.cnt + a0 + lo);
+                cb = __ldg((const unsigned long long*)Q.cnt + jj);
+                tf = (uint32_t)((__ldg(Q.dist + a0 + lo) | __ldg(Q.dist + jj)) >> 15) |
+                     (uint32_t)(__umul64hi(ca, cb) != 0);
+            }
+            if (dsum < best) {
+                best = dsum;
+                sum = 0;
+                flag = 0;
+            }
+            add_term(sum, flag, ca * cb, tf);
+        }
+        if (__shfl_sync(0xFFFFFFFFu, w[kWordUnroll - 1], 31) > end) {  // this step passed hi (or the label's end)
+            uint32_t n = 0;
+#pragma unroll
+            for (int k = 0; k < kWordUnroll; ++k) n += __popc(__ballot_sync(0xFFFFFFFFu, w[k] <= end && w[k] != kNoHub));
+            return j + n;
+        }
+    }
+    return je;
+}
+
+// The warp's minimum, and the sum over the lanes at it, in every lane.
+__device__ __forceinline__ void warp_total(uint32_t& best, uint64_t& sum, uint32_t& flag) {
+    const uint32_t m = __reduce_min_sync(0xFFFFFFFFu, best);
+    if (best != m) {
+        sum = 0;
+        flag = 0;
+    }
+    best = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t os = __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        const uint32_t of = __shfl_xor_sync(0xFFFFFFFFu, flag, o);
+        add_term(sum, flag, os, of);
+    }
+}
+
+__device__ __forceinline__ void write_answer(const QueryArgs& Q, int64_t p, uint32_t best, uint64_t sum, uint32_t flag) {
+    if (best == 0xFFFFFFFFu) {
+        write_fixed(Q, p, PSPC_UNREACHED, 0);
+        return;
+    }
+    Q.out_dist[p] = (uint16_t)best;
+    Q.out_cnt[p] = sum;
+    if (Q.out_ovf) Q.out_ovf[p] = (uint8_t)(flag != 0);
+}
+
+__global__ void __launch_bounds__(kQueryThreads, 5) k_query_words(const QueryArgs Q, int per) {
+    extern __shared__ __align__(16) uint32_t qtab[];
+    const unsigned FULL = 0xFFFFFFFFu;
+    const uint32_t kNone = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t* tab = qtab + w * kWordBuckets * 4;
+    const int64_t nwarps = (int64_t)gridDim.x * (kQueryThreads / 32);
+    const int64_t chunks = (Q.q + per - 1) / per;
+    for (int64_t chunk = (int64_t)blockIdx.x * (kQueryThreads / 32) + w; chunk < chunks; chunk += nwarps) {
+        // a lane's pair, and its answer so far
+        const int64_t k = chunk * per + lane;
+        int64_t p = -1, a0 = 0, b0 = 0;
+        int32_t s = -1;
+        uint32_t la = 0, lb = 0, next = 0;  // next: entries of L(t) done with
+        uint32_t best = kNone, flag = 0;
+        uint64_t sum = 0;
+        bool open = false;
+        if (lane < per && k < Q.q) {
+            p = Q.perm ? (int64_t)__ldg(Q.perm + k) : k;
+            s = __ldg(Q.pairs + 2 * p);
+            const int32_t t = __ldg(Q.pairs + 2 * p + 1);
+            if (s < 0 || s >= Q.n || t < 0 || t >= Q.n) {
+                atomicOr(Q.err, 1);
+                write_fixed(Q, p, PSPC_UNREACHED, 0);
+            } else if (s == t) {
+                write_fixed(Q, p, 0, 1);
+            } else {
+                const int32_t rs = __ldg(Q.rank + s), rt = __ldg(Q.rank + t);
+                a0 = __ldg(Q.off + rs);
+                la = (uint32_t)(__ldg(Q.off + rs + 1) - a0);
+                b0 = __ldg(Q.off + rt);
+                lb = (uint32_t)(__ldg(Q.off + rt + 1) - b0);
+                open = true;
+            }
+        }
+        unsigned todo = __ballot_sync(FULL, open);
+        while (todo) {
+            const int lead = __ffs(todo) - 1;
+            const int32_t source = __shfl_sync(FULL, s, lead);
+            unsigned group = __ballot_sync(FULL, open && s == source);
+            todo &= ~group;
+            int64_t ga = __shfl_sync(FULL, a0, lead);
+            uint32_t gla = __shfl_sync(FULL, la, lead);
+            if (!(group & (group - 1))) {  // one pair: the shorter label goes into the hash
+                if (__shfl_sync(FULL, lb, lead) < gla) {
+                    const int64_t x = a0;
+                    const uint32_t y = la;
+                    if (lane == lead) {
+                        a0 = b0;
+                        la = lb;
+                        b0 = x;
+                        lb = y;
+                    }
+                    ga = __shfl_sync(FULL, a0, lead);
+                    gla = __shfl_sync(FULL, la, lead);
+                }
+            }
+            // pairs with one short label: its entries are looked up in the other
+            for (unsigned m = group; m; m &= m - 1) {
+                const int i = __ffs(m) - 1;
+                const int64_t pb = __shfl_sync(FULL, b0, i);
+                const uint32_t plb = __shfl_sync(FULL, lb, i);
+                const bool brief_a = is_brief(gla, plb), brief_b = is_brief(plb, gla);
+                if (!brief_a && !brief_b) continue;
+                group &= ~(1u << i);
+                uint32_t pbest = kNone, pflag = 0;
+                uint64_t psum = 0;
+                if (brief_a) look_up_label(Q, ga, ga + gla, pb, pb + plb, lane, pbest, psum, pflag);
+                else look_up_label(Q, pb, pb + plb, ga, ga + gla, lane, pbest, psum, pflag);
+                warp_total(pbest, psum, pflag);
+                if (lane == i) {
+                    best = pbest;
+                    sum = psum;
+                    flag = pflag;
+                }
+            }
+            const int32_t* A = Q.hub + ga;
+            for (uint32_t i0 = 0; i0 < gla && group; i0 += kWordSegment) {
+                const uint32_t i1 = min(gla, i0 + kWordSegment);
+                fill_words(tab, A, i0, i1, Q.sh, lane);
+                const uint32_t hi = (uint32_t)__ldg(A + i1 - 1) >> Q.sh;
+                for (unsigned m = group; m; m &= m - 1) {
+                    const int i = __ffs(m) - 1;
+                    const int64_t pb = __shfl_sync(FULL, b0, i);
+                    const uint32_t plb = __shfl_sync(FULL, lb, i), pn = __shfl_sync(FULL, next, i);
+                    const uint32_t had = __shfl_sync(FULL, best, i);
+                    uint32_t pbest = had, pflag = 0;
+                    uint64_t psum = 0;
+                    const uint32_t upto = probe_words(Q, tab, ga, i0, i1, pb, pn, plb, hi, lane, pbest, psum, pflag);
+                    warp_total(pbest, psum, pflag);
+                    if (lane == i) {
+                        next = upto;
+                        if (pbest < best) {
+                            best = pbest;
+                            sum = psum;
+                            flag = pflag;
+                        } else {
+                            add_term(sum, flag, psum, pflag);  // 0 where nothing reached the minimum
+                        }
+                    }
+                    if (upto >= plb) group &= ~(1u << i);  // L(t) is done with
+                }
+                __syncwarp();
+            }
+        }
+        if (open) write_answer(Q, p, best, sum, flag);
+    }
+}
+
+// A few unsorted pairs: a CTA each, its warps joining as many parts of the
+// shorter label with the parts of the longer one at the same hubs.
+__global__ void __launch_bounds__(kQueryThreads, 5) k_query_words_split(const QueryArgs Q) {
+    extern __shared__ __align__(16) uint32_t qtab[];
+    constexpr int kWarps = kQueryThreads / 32;
+    __shared__ uint32_t s_best[kWarps], s_flag[kWarps];
+    __shared__ uint64_t s_sum[kWarps];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t* tab = qtab + w * kWordBuckets * 4;
+    for (int64_t k = blockIdx.x; k < Q.q; k += gridDim.x) {
+        const int64_t p = Q.perm ? (int64_t)__ldg(Q.perm + k) : k;
+        const int32_t s = __ldg(Q.pairs + 2 * p), t = __ldg(Q.pairs + 2 * p + 1);
+        const bool valid = s >= 0 && s < Q.n && t >= 0 && t < Q.n;
+        if (!valid || s == t) {
+            if (threadIdx.x == 0) {
+                if (!valid) atomicOr(Q.err, 1);
+                write_fixed(Q, p, valid ? (uint16_t)0 : (uint16_t)PSPC_UNREACHED, valid ? 1 : 0);
+            }
+            continue;
+        }
+        const int32_t rs = __ldg(Q.rank + s), rt = __ldg(Q.rank + t);
+        int64_t a0 = __ldg(Q.off + rs), b0 = __ldg(Q.off + rt);
+        uint32_t la = (uint32_t)(__ldg(Q.off + rs + 1) - a0), lb = (uint32_t)(__ldg(Q.off + rt + 1) - b0);
+        if (la > lb) {
+            const int64_t x = a0;
+            const uint32_t y = la;
+            a0 = b0;
+            la = lb;
+            b0 = x;
+            lb = y;
+        }
+        uint32_t best = 0xFFFFFFFFu, flag = 0;
+        uint64_t sum = 0;
+        if (la <= 64) {
+            if (w == 0) look_up_label(Q, a0, a0 + la, b0, b0 + lb, lane, best, sum, flag);
+        } else {
+            const uint32_t f0 = (uint32_t)((uint64_t)la * w / kWarps), f1 = (uint32_t)((uint64_t)la * (w + 1) / kWarps);
+            uint32_t lo = 0, hi = lb;  // L(t) from the part's first hub on
+            const uint32_t from = (uint32_t)__ldg(Q.hub + a0 + f0) >> Q.sh;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (((uint32_t)__ldg(Q.hub + b0 + mid) >> Q.sh) < from) lo = mid + 1; else hi = mid;
+            }
+            for (uint32_t i0 = f0; i0 < f1 && lo < lb; i0 += kWordSegment) {
+                const uint32_t i1 = min(f1, i0 + kWordSegment);
+                fill_words(tab, Q.hub + a0, i0, i1, Q.sh, lane);
+                lo = probe_words(Q, tab, a0, i0, i1, b0, lo, lb, (uint32_t)__ldg(Q.hub + a0 + i1 - 1) >> Q.sh, lane, best,
+                                 sum, flag);
+                __syncwarp();
+            }
+        }
+        warp_total(best, sum, flag);
+        if (lane == 0) {
+            s_best[w] = best;
+            s_sum[w] = sum;
+            s_flag[w] = flag;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k2 = 1; k2 < kWarps; ++k2) {
+                if (s_best[k2] > best || s_best[k2] == 0xFFFFFFFFu) continue;
+                if (s_best[k2] < best) {
+                    best = s_best[k2];
+                    sum = 0;
+                    flag = 0;
+                }
+                add_term(sum, flag, s_sum[k2], s_flag[k2]);
+            }
+            write_answer(Q, p, best, sum, flag);
+        }
+        __syncthreads();
+    }
+}
+
+// The same for an index without such words: hubs and distances from their
+// own arrays, counts at every match that reaches a lane's minimum.
 constexpr int kChunkWarps = kQueryThreads / 32;
 
 // At most 40 registers, so that 6 CTAs (48 warps) fit an SM: the kernel
@@ -348,7 +686,7 @@ __global__ void __launch_bounds__(kBySourceThreads) k_query_by_source(const Quer
             for (uint32_t i = tid; i < slots; i += blockDim.x) tab[i] = kEmptySlot;
             __syncthreads();
             for (uint32_t i = tid; i < la; i += blockDim.x) {
-                const uint32_t h = (uint32_t)__ldg(Q.hub + a0 + i);
+                const uint32_t h = (uint32_t)__ldg(Q.hub + a0 + i) >> Q.sh;
                 const unsigned long long v = (unsigned long long)h | ((unsigned long long)__ldg(Q.dist + a0 + i) << 24) |
                                              ((unsigned long long)i << 40);
                 uint32_t slot = hash_hub(h) & mask;
@@ -384,7 +722,7 @@ __global__ void __launch_bounds__(kBySourceThreads) k_query_by_source(const Quer
 #pragma unroll
                     for (int u = 0; u < kBySourceUnroll; ++u) {
                         const int64_t j = j0 + 32 * u + lane;
-                        hb[u] = j < lb ? (uint32_t)__ldg(Q.hub + b0 + j) : kNoHub;
+                        hb[u] = j < lb ? (uint32_t)__ldg(Q.hub + b0 + j) >> Q.sh : kNoHub;
                         db[u] = j < lb ? __ldg(Q.dist + b0 + j) : (uint16_t)0;
                     }
 #pragma unroll
@@ -425,7 +763,9 @@ __global__ void __launch_bounds__(kBySourceThreads) k_query_by_source(const Quer
 }
 
 // One step of L(t) for a lane: entries j0 + 32 u + lane (hub kNoHub past
-// the end of the label).
+// the end of the label). kWords: words of an index that has them, which hold
+// the distance (db is not read).
+template <bool kWords>
 __device__ __forceinline__ void load_step(const int32_t* __restrict__ hubt, const uint16_t* __restrict__ distt,
                                           uint32_t j0, uint32_t lb, int lane, uint32_t (&hb)[kBySourceUnroll],
                                           uint32_t (&db)[kBySourceUnroll]) {
@@ -433,14 +773,14 @@ __device__ __forceinline__ void load_step(const int32_t* __restrict__ hubt, cons
 #pragma unroll
         for (int u = 0; u < kBySourceUnroll; ++u) {
             hb[u] = (uint32_t)__ldg(hubt + j0 + 32 * u + lane);
-            db[u] = __ldg(distt + j0 + 32 * u + lane);
+            db[u] = kWords ? 0u : __ldg(distt + j0 + 32 * u + lane);
         }
     } else {
 #pragma unroll
         for (int u = 0; u < kBySourceUnroll; ++u) {
             const uint32_t j = j0 + 32 * u + lane;
             hb[u] = j < lb ? (uint32_t)__ldg(hubt + j) : kNoHub;
-            db[u] = j < lb ? __ldg(distt + j) : 0u;
+            db[u] = !kWords && j < lb ? __ldg(distt + j) : 0u;
         }
     }
 }
@@ -459,15 +799,18 @@ constexpr uint32_t kBySourceCand = 256;
 
 // Adds the count products of the warp's list to the lanes' partial sums:
 // lane i takes entries i, i + 32, ..., so the loads are independent.
+template <bool kWords>
 __device__ __forceinline__ void add_candidates(const QueryArgs& Q, int64_t a0, const unsigned long long* cntt,
-                                               const uint32_t* cw, uint32_t nc, int lane, uint64_t& sum,
+                                               const uint16_t* distt, const uint32_t* cw, uint32_t nc, int lane, uint64_t& sum,
                                                uint32_t& flag) {
     __syncwarp();
     for (uint32_t c = lane; c < nc; c += 32) {
         const uint32_t v = cw[c];
         const uint64_t ca = __ldg((const unsigned long long*)Q.cnt + a0 + ((v >> 1) & 0x7FFFu));
         const uint64_t cb = __ldg(cntt + (v >> 16));
-        add_term(sum, flag, ca * cb, (v & 1u) | (uint32_t)(__umul64hi(ca, cb) != 0));
+        const uint32_t f = kWords ? (uint32_t)(__ldg(Q.dist + a0 + ((v >> 1) & 0x7FFFu)) | __ldg(distt + (v >> 16))) >> 15
+                                  : v & 1u;
+        add_term(sum, flag, ca * cb, f | (uint32_t)(__umul64hi(ca, cb) != 0));
     }
     __syncwarp();
 }
@@ -489,7 +832,10 @@ __device__ __forceinline__ void add_candidates(const QueryArgs& Q, int64_t a0, c
 // minimum join a per-warp list in shared memory. Counts are read only for
 // the list, once per pair (or when it fills), all loads independent: reads
 // at every match that reached a lane's minimum so far cost one 32-byte
-// sector each and one load round trip each inside the stream.
+// sector each and one load round trip each inside the stream. On an index
+// with words the stream is the words alone, and the flags are read with the
+// counts.
+template <bool kWords>
 __global__ void __launch_bounds__(kBySourceThreads)
     k_query_by_source_direct(const QueryArgs Q, uint32_t n_pad, uint32_t label_pad) {
     extern __shared__ uint16_t dsm[];
@@ -497,6 +843,7 @@ __global__ void __launch_bounds__(kBySourceThreads)
     uint16_t* sd = dsm + n_pad;  // entries of the largest label (label_pad: even)
     __shared__ unsigned long long s_next;
     const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t dmask = (1u << Q.db) - 1u;
     uint32_t* cw = (uint32_t*)(dsm + n_pad + label_pad) + (tid >> 5) * kBySourceCand;  // the warp's list
     for (uint32_t i = tid; i < n_pad; i += blockDim.x) pos[i] = 0xFFFFu;
     __syncthreads();
@@ -528,8 +875,9 @@ __global__ void __launch_bounds__(kBySourceThreads)
             const int64_t a0 = __ldg(Q.off + rs);
             const uint32_t la = (uint32_t)(__ldg(Q.off + rs + 1) - a0);
             for (uint32_t i = tid; i < la; i += blockDim.x) {
-                pos[__ldg(Q.hub + a0 + i)] = (uint16_t)i;
-                sd[i] = __ldg(Q.dist + a0 + i);
+                const uint32_t w = (uint32_t)__ldg(Q.hub + a0 + i);
+                pos[kWords ? w >> Q.sh : w] = (uint16_t)i;
+                sd[i] = kWords ? (uint16_t)(w >> Q.cb & dmask) : __ldg(Q.dist + a0 + i);
             }
             if (tid == 0) s_next = (unsigned long long)r0;
             __syncthreads();
@@ -565,7 +913,7 @@ __global__ void __launch_bounds__(kBySourceThreads)
                 // loads are in flight while this step probes
                 const uint32_t lbu = (uint32_t)lb;
                 uint32_t nh[kBySourceUnroll], nd[kBySourceUnroll];
-                load_step(hubt, distt, 0, lbu, lane, nh, nd);
+                load_step<kWords>(hubt, distt, 0, lbu, lane, nh, nd);
                 for (uint32_t j0 = 0; j0 < lbu; j0 += 32 * kBySourceUnroll) {
                     uint32_t hb[kBySourceUnroll], db[kBySourceUnroll];
 #pragma unroll
@@ -573,13 +921,14 @@ __global__ void __launch_bounds__(kBySourceThreads)
                         hb[u] = nh[u];
                         db[u] = nd[u];
                     }
-                    if (j0 + 32 * kBySourceUnroll < lbu) load_step(hubt, distt, j0 + 32 * kBySourceUnroll, lbu, lane, nh, nd);
+                    if (j0 + 32 * kBySourceUnroll < lbu) load_step<kWords>(hubt, distt, j0 + 32 * kBySourceUnroll, lbu, lane, nh, nd);
                     // key of a match: distance sum << 16 | L(s) position (15 bits) << 1 | a factor's flag
                     uint32_t key[kBySourceUnroll];
                     uint32_t kmin = 0xFFFFFFFFu;
 #pragma unroll
                     for (int u = 0; u < kBySourceUnroll; ++u) {
-                        const uint32_t ia = hb[u] == kNoHub ? 0xFFFFu : (uint32_t)pos[hb[u]];
+                        const uint32_t ia = hb[u] == kNoHub ? 0xFFFFu : (uint32_t)pos[kWords ? hb[u] >> Q.sh : hb[u]];
+                        if (kWords) db[u] = hb[u] >> Q.cb & dmask;
                         const uint32_t da = ia == 0xFFFFu ? 0u : (uint32_t)sd[ia];
                         key[u] = ia == 0xFFFFu ? 0xFFFFFFFFu
                                                : ((da & 0x7FFFu) + (db[u] & 0x7FFFu)) << 16 | ia << 1 | ((da | db[u]) >> 15);
@@ -602,7 +951,7 @@ __global__ void __launch_bounds__(kBySourceThreads)
                         const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
                         if (m == 0) continue;
                         if (nc + (uint32_t)__popc(m) > kBySourceCand) {  // rare: a full list
-                            add_candidates(Q, a0, cntt, cw, nc, lane, sum, flag);
+                            add_candidates<kWords>(Q, a0, cntt, distt, cw, nc, lane, sum, flag);
                             nc = 0;
                         }
                         if (hit)
@@ -611,11 +960,11 @@ __global__ void __launch_bounds__(kBySourceThreads)
                         nc += (uint32_t)__popc(m);
                     }
                 }
-                add_candidates(Q, a0, cntt, cw, nc, lane, sum, flag);
+                add_candidates<kWords>(Q, a0, cntt, distt, cw, nc, lane, sum, flag);
                 finish_pair_warp(Q, p, best == 0xFFFFu ? 0xFFFFFFFFu : best, sum, flag, lane);
             }
             __syncthreads();
-            for (uint32_t i = tid; i < la; i += blockDim.x) pos[__ldg(Q.hub + a0 + i)] = 0xFFFFu;
+            for (uint32_t i = tid; i < la; i += blockDim.x) pos[(uint32_t)__ldg(Q.hub + a0 + i) >> (kWords ? Q.sh : 0)] = 0xFFFFu;
             __syncthreads();
             r0 = r1;
         }
@@ -662,9 +1011,14 @@ static void set_query_carveouts() {
         prefer_max_shared((const void*)k_query_by_source);
         cudaFuncSetAttribute((const void*)k_query_by_source, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kBySourceMaxSlots * 8));
-        prefer_max_shared((const void*)k_query_by_source_direct);
-        cudaFuncSetAttribute((const void*)k_query_by_source_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kBySourceDirectBytes);
+        for (const void* f : {(const void*)k_query_words, (const void*)k_query_words_split}) {
+            prefer_max_shared(f);
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordBytes);
+        }
+        for (const void* f : {(const void*)k_query_by_source_direct<false>, (const void*)k_query_by_source_direct<true>}) {
+            prefer_max_shared(f);
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBySourceDirectBytes);
+        }
         prefer_max_shared((const void*)k_query<8>);
         prefer_max_shared((const void*)k_query<16>);
         prefer_max_shared((const void*)k_query<32>);
@@ -698,14 +1052,36 @@ static size_t by_source_direct_bytes(const Index& ix) {
     return b + (size_t)(kBySourceThreads / 32) * kBySourceCand * 4 <= kBySourceDirectBytes ? b : 0;
 }
 
-// The query kernel. Automatic choice: by source when the pairs are grouped,
-// L(s) fits on chip and sources repeat often (q >= 64 n: each table build
-// serves many pairs; with fewer pairs per source the staged merge-join,
-// whose L(s) reads mostly hit L2 after the grouping sort, measured faster);
-// otherwise lanes per pair from the label sizes: wide groups for long
-// labels (fewer merge steps), narrow groups for short ones (more pairs in
-// flight per warp), warp-staged chunks of 256 entries for long labels.
+// The query kernel. Automatic choice: on an index with words, for labels of 24
+// entries or more on average, the words query: a warp per few pairs, or a CTA
+// per pair for few pairs with long labels. On the others by source when the
+// pairs are grouped, L(s) fits on chip and sources repeat often (q >= 64 n:
+// each table build serves many pairs; with fewer pairs per source the staged
+// merge-join, whose L(s) reads mostly hit L2 after the grouping sort, measured
+// faster); otherwise lanes per pair from the label sizes: wide groups for
+// long labels (fewer merge steps), narrow groups for short ones (more pairs
+// in flight per warp), warp-staged chunks of 256 entries for long labels.
+constexpr int kQueryWords = 3;
+// Measured (GB300): 10^6 pairs on R-MAT 65,536 5.21 -> 2.77 ms, 4x10^6 on R-MAT
+// 262,144 24.4 -> 12.1 ms, 10^6 on BA 2,000 (97 entries) 1.01 -> 0.73 ms.
+constexpr int64_t kWordsLabel = 24;
+// Runs of 64 or more pairs of one source with long labels stay with the
+// table of positions, which is filled once a run: 10^7 pairs on R-MAT 65,536
+// 16.4 against 23.4 ms, 2x10^6 on BA 20,011 (545 entries) 3.2 against 4.7; with
+// labels of 128 entries it loses (R-MAT 8,000: 1.62 against 1.41 ms).
+constexpr int64_t kRunsLabel = 256;
+// Pairs per vertex from which they are sorted by source (3 of them: 0.82 ms
+// sorted, 1.00 not; 1: 0.42 and 0.36, R-MAT 65,536).
+constexpr int64_t kWordsSort = 2;
+// Pairs up to which a CTA per pair pays, from this average label on (R-MAT
+// 262,144: 1,500 pairs 43 us, with a warp each 90; 4,000 80 against 122 for the
+// staged chunks; 20,000 422 against 264).
+constexpr int64_t kWordsSplit = 4096;
+constexpr int64_t kWordsSplitLabel = 128;
 static int query_group_for(const Index& ix, bool grouped, int64_t q) {
+    if (ix.db && ix.query_group >= 64) return kQueryWords;
+    const bool runs = grouped && q >= 64 * ix.n && by_source_direct_bytes(ix) > 0 && ix.entries >= kRunsLabel * ix.n;
+    if (ix.db && ix.query_group == 0 && ix.entries >= kWordsLabel * ix.n && !runs) return kQueryWords;
     const bool by_source_ok = grouped && (by_source_direct_bytes(ix) > 0 || by_source_slots(ix) > 0);
     if (ix.query_group == PSPC_QUERY_BY_SOURCE && by_source_ok) return PSPC_QUERY_BY_SOURCE;
     if (ix.query_group == PSPC_QUERY_BY_SOURCE_HASH && grouped && by_source_slots(ix) > 0)
@@ -713,6 +1089,7 @@ static int query_group_for(const Index& ix, bool grouped, int64_t q) {
     if (ix.query_group && ix.query_group != PSPC_QUERY_BY_SOURCE && ix.query_group != PSPC_QUERY_BY_SOURCE_HASH)
         return ix.query_group;
     if (ix.query_group == 0 && by_source_ok && q >= 64 * ix.n) return PSPC_QUERY_BY_SOURCE;
+    if (ix.db && ix.entries >= kWordsLabel * ix.n) return kQueryWords;  // the staged chunks read plain hubs
     const double avg = ix.n ? (double)ix.entries / (double)ix.n : 0.0;
     return avg >= 128.0 ? 256 : (avg >= 24.0 ? 16 : 8);
 }
@@ -721,6 +1098,12 @@ static int query_group_for(const Index& ix, bool grouped, int64_t q) {
 // pspc_query_noalloc): when sources repeat enough for L(s) to be reused.
 static bool groups_by_source(const Index& ix, int64_t q) {
     return q >= 4096 && q >= ix.n / 4 && q < ((int64_t)1 << 31);
+}
+
+// The words query profits from the order only where a source has several
+// pairs: below that its sort costs more than it saves.
+static bool sorts_by_source(const Index& ix, int64_t q) {
+    return groups_by_source(ix, q) && (query_group_for(ix, true, q) != kQueryWords || q >= kWordsSort * ix.n);
 }
 
 // Launches the query kernel chosen for the index (Q.perm is the grouping
@@ -732,18 +1115,36 @@ static cudaError_t launch_query(Index& ix, const QueryArgs& Q, cudaStream_t st) 
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ix.device);
     if (e != cudaSuccess) return e;
     __atomic_fetch_add(&ix.query_launches, (int64_t)1, __ATOMIC_RELAXED);
+    if (G == kQueryWords) {
+        const bool split = Q.q <= kWordsSplit && ix.entries >= kWordsSplitLabel * ix.n;
+        const void* f = split ? (const void*)k_query_words_split : (const void*)k_query_words;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kQueryThreads, kWordBytes);
+        if (e != cudaSuccess) return e;
+        const int64_t ctas = (int64_t)sms * std::max(occ, 1), warps = ctas * (kQueryThreads / 32);
+        if (split) {
+            k_query_words_split<<<(int)std::min<int64_t>(Q.q, ctas), kQueryThreads, kWordBytes, st>>>(Q);
+            return cudaGetLastError();
+        }
+        // up to 32 pairs to a warp, but four turns for every warp
+        const int per = (int)std::max<int64_t>(1, std::min<int64_t>(32, Q.q / (warps * 4)));
+        const int64_t want = ((Q.q + per - 1) / per + kQueryThreads / 32 - 1) / (kQueryThreads / 32);
+        k_query_words<<<(int)std::max<int64_t>(1, std::min(want, ctas)), kQueryThreads, kWordBytes, st>>>(Q, per);
+        return cudaGetLastError();
+    }
     if (G == PSPC_QUERY_BY_SOURCE && by_source_direct_bytes(ix) > 0) {
         // positions above a ninth of the shared memory leave room for one CTA
         // per SM: make it a large one; smaller tables share SMs
         const size_t base = by_source_direct_bytes(ix);
         const int threads = base > (size_t)24 * 1024 ? kBySourceThreads : kQueryThreads;
         const size_t smem = base + (size_t)(threads / 32) * kBySourceCand * 4;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k_query_by_source_direct, threads, smem);
+        const void* f = ix.db ? (const void*)k_query_by_source_direct<true> : (const void*)k_query_by_source_direct<false>;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, threads, smem);
         if (e != cudaSuccess) return e;
         const int64_t items = (Q.q + kBySourceItem - 1) / kBySourceItem;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, (int64_t)sms * std::max(occ, 1)));
-        k_query_by_source_direct<<<grid, threads, smem, st>>>(Q, (uint32_t)((ix.n + 1) & ~(int64_t)1),
-                                                             by_source_label_pad(ix));
+        const uint32_t n_pad = (uint32_t)((ix.n + 1) & ~(int64_t)1), l_pad = by_source_label_pad(ix);
+        if (ix.db) k_query_by_source_direct<true><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
+        else k_query_by_source_direct<false><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
         return cudaGetLastError();
     }
     if (G == PSPC_QUERY_BY_SOURCE || G == PSPC_QUERY_BY_SOURCE_HASH) {
@@ -893,7 +1294,7 @@ extern "C" int pspc_query(const pspc_index* hc, const int32_t* pairs, int64_t q,
     // Group by source when sources repeat enough for L(s) to be reused.
     int32_t* d_perm = nullptr;
     int64_t* d_bins = nullptr;
-    const bool group = groups_by_source(ix, q);
+    const bool group = sorts_by_source(ix, q);
     if (e == cudaSuccess && group) {
         const int32_t* pin = dev_in ? pairs : d_pairs;
         e = dev_alloc((void**)&d_perm, (size_t)q * 4, st);
@@ -923,6 +1324,9 @@ extern "C" int pspc_query(const pspc_index* hc, const int32_t* pairs, int64_t q,
         Q.rank = ix.rank;
         Q.off = ix.off;
         Q.hub = ix.hub;
+        Q.sh = ix.sh;
+        Q.cb = ix.cb;
+        Q.db = ix.db;
         Q.dist = ix.dist;
         Q.cnt = ix.cnt;
         Q.pairs = dev_in ? pairs : d_pairs;
@@ -1056,6 +1460,9 @@ extern "C" int pspc_query_noalloc(const pspc_index* hc, const int32_t* pairs, in
             Q.rank = ix.rank;
             Q.off = ix.off;
             Q.hub = ix.hub;
+            Q.sh = ix.sh;
+            Q.cb = ix.cb;
+            Q.db = ix.db;
             Q.dist = ix.dist;
             Q.cnt = ix.cnt;
             Q.pairs = pairs;
@@ -1102,6 +1509,9 @@ extern "C" int pspc_query_async(const pspc_index* hc, const int32_t* pairs, int6
     Q.rank = ix.rank;
     Q.off = ix.off;
     Q.hub = ix.hub;
+    Q.sh = ix.sh;
+    Q.cb = ix.cb;
+    Q.db = ix.db;
     Q.dist = ix.dist;
     Q.cnt = ix.cnt;
     Q.pairs = pairs;

@@ -319,7 +319,7 @@ extern "C" int pspc_export(const pspc_index* h, int64_t* off, int32_t* hub, uint
             off[v] = p;
             const int32_t r = rank[v];
             for (int64_t i = roff[r]; i < roff[r + 1]; ++i, ++p) {
-                hub[p] = order[rhub[i]];
+                hub[p] = order[(uint32_t)rhub[i] >> ix.sh];
                 dist[p] = (uint16_t)(rdist[i] & 0x7FFF);
                 ovf[p] = (uint8_t)(rdist[i] >> 15);
                 cnt[p] = rcnt[i];
@@ -337,7 +337,7 @@ extern "C" int pspc_export(const pspc_index* h, int64_t* off, int32_t* hub, uint
 namespace pspc {
 
 // Thread per (rank-space) vertex: binary search of the hub in its sorted label.
-__global__ void k_hub_column(int64_t n, int32_t rw, const int32_t* __restrict__ order, const int64_t* __restrict__ off,
+__global__ void k_hub_column(int64_t n, int32_t rw, int sh, const int32_t* __restrict__ order, const int64_t* __restrict__ off,
                              const int32_t* __restrict__ hub, const uint16_t* __restrict__ dist,
                              const uint64_t* __restrict__ cnt, uint16_t* out_dist, uint64_t* out_cnt,
                              uint8_t* out_ovf) {
@@ -347,10 +347,10 @@ __global__ void k_hub_column(int64_t n, int32_t rw, const int32_t* __restrict__ 
     const int64_t e = hi;
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
-        if (hub[mid] < rw) lo = mid + 1; else hi = mid;
+        if (((uint32_t)hub[mid] >> sh) < (uint32_t)rw) lo = mid + 1; else hi = mid;
     }
     const int32_t v = order[r];
-    if (lo < e && hub[lo] == rw) {
+    if (lo < e && ((uint32_t)hub[lo] >> sh) == (uint32_t)rw) {
         out_dist[v] = (uint16_t)(dist[lo] & 0x7FFF);
         out_cnt[v] = cnt[lo];
         out_ovf[v] = (uint8_t)(dist[lo] >> 15);
@@ -378,7 +378,7 @@ __global__ void k_vert_sizes(int64_t k, const int32_t* __restrict__ verts, int64
 // Warp per selected vertex: its label with hubs as caller ids.
 __global__ void k_vert_gather(int64_t k, const int32_t* __restrict__ verts, int64_t n, const int32_t* __restrict__ rank,
                               const int32_t* __restrict__ order, const int64_t* __restrict__ off,
-                              const int32_t* __restrict__ hub, const uint16_t* __restrict__ dist,
+                              const int32_t* __restrict__ hub, int sh, const uint16_t* __restrict__ dist,
                               const uint64_t* __restrict__ cnt, const int64_t* __restrict__ pos, int32_t* o_hub,
                               uint16_t* o_dist, uint64_t* o_cnt, uint8_t* o_ovf) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -389,7 +389,7 @@ __global__ void k_vert_gather(int64_t k, const int32_t* __restrict__ verts, int6
     const int32_t r = rank[v];
     const int64_t a0 = off[r], len = off[r + 1] - a0, p0 = pos[i];
     for (int64_t j = lane; j < len; j += 32) {
-        o_hub[p0 + j] = order[hub[a0 + j]];
+        o_hub[p0 + j] = order[(uint32_t)hub[a0 + j] >> sh];
         o_dist[p0 + j] = (uint16_t)(dist[a0 + j] & 0x7FFF);
         o_ovf[p0 + j] = (uint8_t)(dist[a0 + j] >> 15);
         o_cnt[p0 + j] = cnt[a0 + j];
@@ -415,7 +415,7 @@ extern "C" int pspc_hub_column(const pspc_index* h, int32_t w, uint16_t* dist, u
     if (e == cudaSuccess) e = dev_alloc((void**)&d_cnt, ix.n * 8, st);
     if (e == cudaSuccess) e = dev_alloc((void**)&d_ovf, ix.n, st);
     if (e == cudaSuccess) {
-        k_hub_column<<<(unsigned)((ix.n + 255) / 256), 256, 0, st>>>(ix.n, rw, ix.order, ix.off, ix.hub, ix.dist,
+        k_hub_column<<<(unsigned)((ix.n + 255) / 256), 256, 0, st>>>(ix.n, rw, ix.sh, ix.order, ix.off, ix.hub, ix.dist,
                                                                       ix.cnt, d_dist, d_cnt, d_ovf);
         e = cudaGetLastError();
     }
@@ -478,7 +478,7 @@ extern "C" int pspc_export_vertices(const pspc_index* h, const int32_t* verts, i
             if (e == cudaSuccess) e = dev_alloc((void**)&d_ovf, E, st);
             if (e == cudaSuccess) {
                 k_vert_gather<<<(unsigned)((k * 32 + 255) / 256), 256, 0, st>>>(
-                    k, d_verts, ix.n, ix.rank, ix.order, ix.off, ix.hub, ix.dist, ix.cnt, d_pos, d_hub, d_dist, d_cnt,
+                    k, d_verts, ix.n, ix.rank, ix.order, ix.off, ix.hub, ix.sh, ix.dist, ix.cnt, d_pos, d_hub, d_dist, d_cnt,
                     d_ovf);
                 e = cudaGetLastError();
             }

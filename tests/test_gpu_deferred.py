@@ -1,0 +1,45 @@
+"""Deep levels' label scans, queued and run by later launches: the index
+equals the oracle's with so few landmarks that most candidates are undecided
+and many are pruned by their scans (segments closed with entries taken out),
+with more undecided candidates than the queue holds, for the warp-per-vertex
+and the CTA-per-vertex kernels, and with few CTAs."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import pspc_inputs as P
+from tests import _graphs as G
+from tests.test_gpu_parity import assert_index_equal, gpu_index, pspc  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name,order", [("grid90", "degree"), ("grid70", "random")])
+def test_deferred_scans(pspc, name, order):  # noqa: F811
+    g, rank, _ = P.workload(name)
+    if order == "random":
+        rank = G.random_rank(g.n, 9)
+    ref = oracle.OracleIndex(g, rank).export()
+    for kw in (dict(landmarks=1), dict(landmarks=1, warp_levels=-1), dict(landmarks=40, max_ctas=2), dict(granular=True),
+               dict(landmarks=3, arena_entries=1)):
+        ix = gpu_index(pspc, g, rank, **kw)
+        assert_index_equal(ix, ref)
+        ls = ix.level_stats()
+        assert sum(l["entries"] for l in ls) + g.n == len(ref.hub)
+        ix.free()
+
+
+def test_odd_cycles(pspc):  # noqa: F811
+    """Not bipartite: witnesses at both distance sums d-1 and d-2."""
+    rng = np.random.default_rng(3)
+    base = G.grid(64)
+    extra = np.array([(v, v + 65) for v in rng.integers(0, 62 * 64, 700) if v % 64 < 63])
+    g = P.csr_from_edges(base.n, np.concatenate([base.edges(), extra]), "diagonals")
+    rank = P.degree_rank(g, "random", 5)
+    ref = oracle.OracleIndex(g, rank).export()
+    for kw in (dict(), dict(landmarks=2), dict(landmarks=2, warp_levels=-1)):
+        ix = gpu_index(pspc, g, rank, **kw)
+        assert_index_equal(ix, ref)
+        ix.free()
