@@ -26,6 +26,10 @@
 namespace pspc {
 
 constexpr int kFinThreads = 256;
+// What a step of the distance balls costs, and what rule 2 costs a candidate
+// at level 3 (the marking walk) and below it (landmark filter and scans).
+constexpr double kBallStepSeconds = 10e-6, kBallBytesPerSecond = 8e12;
+constexpr double kRule2Level3 = 0.5e-10, kRule2Deeper = 1.2e-10;
 constexpr int kFinSmemKeys = 8192;  // labels up to this size are merged on chip
 
 // ---------------------------------------------------------------------------
@@ -668,6 +672,18 @@ struct Builder {
     int64_t* raw_u = nullptr;
     int64_t* lab_size = nullptr;
     int32_t* items = nullptr;
+    // distance balls (pspc_ball.cu)
+    std::vector<int64_t> graph_n, graph_arcs;  // of a batch's graphs
+    int64_t* ball_off = nullptr;     // batches: first word of every vertex's row [n+1]
+    uint32_t* ball[2] = {nullptr, nullptr};
+    int2* ball_slices = nullptr;
+    int* ball_count = nullptr;
+    int n_ball_slices = 0;
+    int ball_dist = 0;               // distance of ball[0] (0: none yet)
+    int64_t ball_words = 0, ball_row_words = 0;  // of one ball, and of its longest row
+    double ball_step_bytes = 0.0;    // read and written by one step
+    bool ball_level = false;         // the current level has its ball
+    double dup_ratio = 1.0;          // candidates per pulled entry at the last level without one
     HeldSegment* held = nullptr;     // deferred scans: one segment per vertex at most, and the queue
     DeferredScan* scans = nullptr;   // (and behind it the scans left after the proof)
     unsigned int scan_cap = 0;
@@ -706,6 +722,11 @@ struct Builder {
         dfree(raw_u, st);
         dfree(lab_size, st);
         dfree(items, st);
+        dfree(ball_off, st);
+        dfree(ball[0], st);
+        dfree(ball[1], st);
+        dfree(ball_slices, st);
+        dfree(ball_count, st);
         dfree(held, st);
         dfree(scans, st);
         dfree(glist, st);
@@ -813,6 +834,8 @@ struct Builder {
             N += G.n;
             A += arcs_g;
             max_comp = std::max(max_comp, G.n);
+            graph_n.push_back(G.n);
+            graph_arcs.push_back(arcs_g);
             if (N > kMaxVertices || A >= ((int64_t)1 << 40)) rc = PSPC_E_INVAL;
         }
         if (rc == PSPC_OK) {
@@ -1029,10 +1052,14 @@ struct Builder {
         A.comp_base = comp_base;
         A.lmk = d <= kMaxDist ? out.lmk : nullptr;  // the filter compares 15-bit distances
         A.lmk_stride = out.lmk_stride;
+        if (ball_level) {
+            A.ball = ball[0];
+            A.ball_rows = {ball_off, ball_row_words};
+        }
         // shallow levels test the first kLmkShallow landmarks only: their
         // short distances seldom prove survival, and half the row is read
         A.lmk_words = d < kLmkDeepLevel ? std::min(out.lmk_stride / 16, 2 * kLmkShallow / 16) : out.lmk_stride / 16;
-        if (d >= kDeferLevel && A.lmk && (int64_t)hstt->n_active * d >= kDeferWork) {
+        if (d >= kDeferLevel && A.lmk && !A.ball && (int64_t)hstt->n_active * d >= kDeferWork) {
             if (!held) {
                 scan_cap = (unsigned)std::min<int64_t>(std::max<int64_t>(4 * n, 1 << 16), 1 << 26);
                 PSPC_TRY_CUDA(dalloc(&held, n, st));
@@ -1265,6 +1292,73 @@ struct Builder {
         return rc;
     }
 
+    // Sizes of a ball and of a step, before the levels.
+    void ball_sizes() {
+        auto row = [](int64_t m) { return (m + 127) / 128 * 4; };
+        if (graph_n.empty()) {
+            ball_row_words = row(n);
+            ball_words = n * ball_row_words;
+            ball_step_bytes = 4.0 * (double)(arcs + 2 * n) * (double)ball_row_words;
+        } else {
+            for (size_t g = 0; g < graph_n.size(); ++g) {
+                const int64_t w = row(graph_n[g]);
+                ball_row_words = std::max(ball_row_words, w);
+                ball_words += graph_n[g] * w;
+                ball_step_bytes += 4.0 * (double)(graph_arcs[g] + 2 * graph_n[g]) * (double)w;
+            }
+        }
+    }
+
+    // Brings the ball to distance d-1 where that costs less than the landmark
+    // filter, the marking walk and the label scans of level d, which pulls
+    // `raw` entries and will have about as many candidates for them as the
+    // last level without a ball. Measured: a step moves its bytes at 8 to 13
+    // TB/s (a segment of all rows stays in L2); rule 2 took 0.06 to 0.22 ns a
+    // candidate on BA graphs of 20,011 and 100,000 vertices, 0.04 to 0.05 on
+    // R-MAT graphs and at level 3. On grid 256x256 a step would cost 375 us
+    // and save 200 a level, so deep graphs keep the filter.
+    int use_ball(int d, long long raw) {
+        ball_level = false;
+        if (d < 3 || ball_words * 4 > kBallBytes) return PSPC_OK;
+        const int steps = d - 1 - std::max(ball_dist, 1);
+        const double cost = (steps + (ball_dist == 0)) * kBallStepSeconds + steps * ball_step_bytes / kBallBytesPerSecond +
+                            (ball_dist == 0 ? ball_words * 4.0 / kBallBytesPerSecond : 0.0);
+        if (cost >= (double)raw * dup_ratio * (d == 3 ? kRule2Level3 : kRule2Deeper)) return PSPC_OK;
+        if (ball_dist == 0) {
+            if (!graph_n.empty()) {
+                std::vector<int64_t> off;
+                off.reserve((size_t)n + 1);
+                int64_t at = 0;
+                for (int64_t m : graph_n) {
+                    const int64_t w = (m + 127) / 128 * 4;
+                    for (int64_t v = 0; v < m; ++v, at += w) off.push_back(at);
+                }
+                off.push_back(at);
+                PSPC_TRY_CUDA(dalloc(&ball_off, n + 1, st));
+                PSPC_TRY_CUDA(cudaMemcpyAsync(ball_off, off.data(), (n + 1) * 8, cudaMemcpyHostToDevice, st));
+                PSPC_TRY_CUDA(cudaStreamSynchronize(st));  // off is a host buffer of this scope
+            }
+            PSPC_TRY_CUDA(dalloc(&ball[0], ball_words, st));
+            PSPC_TRY_CUDA(dalloc(&ball[1], ball_words, st));
+            PSPC_TRY_CUDA(dalloc(&ball_slices, arcs / 128 + 1, st));
+            PSPC_TRY_CUDA(dalloc(&ball_count, 1, st));
+            PSPC_TRY_CUDA(launch_ball_init(n, arcs, rp_r, arc_src, col_r, comp_base, {ball_off, ball_row_words}, ball_words,
+                                           ball[0], ball_slices, ball_count, st));
+            PSPC_TRY_CUDA(cudaMemcpyAsync(&n_ball_slices, ball_count, sizeof(int), cudaMemcpyDeviceToHost, st));
+            PSPC_TRY_CUDA(cudaStreamSynchronize(st));
+            out.launches += 2;
+            ball_dist = 1;
+        }
+        for (; ball_dist < d - 1; ++ball_dist) {
+            PSPC_TRY_CUDA(launch_ball_step(n, rp_r, col_r, {ball_off, ball_row_words}, ball_row_words, ball_slices,
+                                           n_ball_slices, ball[0], ball[1], st));
+            out.launches += 1 + (n_ball_slices > 0);
+            std::swap(ball[0], ball[1]);
+        }
+        ball_level = true;
+        return PSPC_OK;
+    }
+
     // Push paradigm (Algorithm PUSH): bucket offsets from a scan of the
     // per-arc counts of the cost pass, then every arc copies its entries.
     int push_entries(int d) {
@@ -1313,6 +1407,7 @@ struct Builder {
         PSPC_TRY_CUDA(launch_arc_src(rp_r, n, arc_src, st));
         out.launches += 1;
 
+        ball_sizes();
         k_level0<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, hub_arena, cnt_arena, seg);
         out.launches += 1;
         PSPC_TRY_CUDA(cudaGetLastError());
@@ -1380,6 +1475,7 @@ struct Builder {
             // buckets before the level kernel merges them.
             push_level = o.paradigm == 1;
             if (push_level && (rc = push_entries(d))) break;
+            if (plan.dense_occupancy > 0 && (rc = use_ball(d, raw_total))) break;
             if (skip_prefix)  // on the graphs measured, the share saved only fell after its first level
                 prefix_pays = (double)hstt->prefix_skipped >=
                               kDensePrefixMinGain * (double)(hstt->prefix_skipped + hstt->raw_total);
@@ -1453,6 +1549,7 @@ struct Builder {
             for (int b = 0; b < kBuckets; ++b) ovf_attempts += hstt->route_ovf[b];
             ls.routed_vertices = std::max(0LL, (long long)hstt->n_retry - ovf_attempts);
             out.lstats.push_back(ls);
+            if (!ball_level && raw_total > 0) dup_ratio = (double)ls.unique_candidates / (double)raw_total;
             if (o.verbose)
                 fprintf(stderr, "pspc level %d: raw %lld unique %lld entries %lld active %d (off-chip %d) %.3f ms\n",
                         d, raw_total, (long long)hstt->unique_total, added, hstt->n_active, n_off, ms);

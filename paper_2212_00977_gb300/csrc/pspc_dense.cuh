@@ -22,7 +22,8 @@
 // run lengths; at level 4 the landmark filter and the label scans take 57%.
 // The hash it replaces kept tables of more than 4,096 slots in device memory,
 // half of whose sectors missed L2: levels 3 and 4 took 568 and 495 ms, now
-// 238 and 280 ms (the build 1,182 -> 616 ms; BA 100,000, m = 8: 240 -> 171).
+// 238 and 280 ms (the build 1,182 -> 616 ms; BA 100,000, m = 8: 240 -> 171). With
+// a distance ball its row is the window's bitmap and only the pull is left.
 
 // Words of the window's bitmaps.
 constexpr uint32_t kDenseWords = kDenseWindow / 32;
@@ -130,8 +131,9 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
         // Where each window starts in the pulled run of every arc, and in
         // u's own segments of levels d-1 and d-2 (the only ones that a
         // pulled hub can be in): one table for all windows when it fits.
-        const uint64_t own1 = __ldg(A.seg + (int64_t)(d - 1) * n + u);
-        const uint64_t own2 = d > 2 ? __ldg(A.seg + (int64_t)(d - 2) * n + u) : 0ull;
+        const uint32_t* ball = ball_of(A, u);  // with a ball its row stands for both, and for rule 2
+        const uint64_t own1 = ball ? 0ull : __ldg(A.seg + (int64_t)(d - 1) * n + u);
+        const uint64_t own2 = !ball && d > 2 ? __ldg(A.seg + (int64_t)(d - 2) * n + u) : 0ull;
         const bool table = (uint64_t)(deg + 2) * nb <= (uint64_t)kDenseBounds;
         auto arc_run = [&](int r, uint64_t& start, uint32_t& len) {
             len = __ldg(A.cnt_arc + a0 + r);
@@ -168,7 +170,11 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
         int M = 0;
         for (uint32_t w = 0; w < nwin; ++w) {
             const uint32_t w0 = cbase + w * W;
-            {  // members of L_<d(u) in the window
+            if (ball) {
+                const uint32_t row = (span + 31) / 32;  // words of the row over the ids below u
+                for (uint32_t i = tid; i < kDenseWords && w * kDenseWords + i < row; i += NT)
+                    mem[i] = __ldg(ball + w * kDenseWords + i);
+            } else {  // members of L_<d(u) in the window
                 const uint32_t e1 = edge((uint32_t)deg, seg_start(own1), seg_len(own1), w);
                 const uint32_t e2 = edge((uint32_t)deg + 1, seg_start(own2), seg_len(own2), w);
                 const uint32_t n1 = edge((uint32_t)deg, seg_start(own1), seg_len(own1), w + 1) - e1;
@@ -273,7 +279,7 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
         // |L_1(u)| arcs of its row) are walked and the ids met marked in a
         // bitmap over the counts' memory, 32 kDenseWindow ids at a time.
         bool listed = false;  // list[] holds the candidates (else all of the slab)
-        if (d == 3 && M > 0) {
+        if (d == 3 && M > 0 && !ball) {
             const int len1 = (int)seg_len(__ldg(A.seg + n + u));
             const uint32_t from0 = A.hpre ? (uint32_t)__ldg(A.hpre + u) : 0u;  // ids below are members, no candidates
             uint32_t* mk = acc;
@@ -351,7 +357,7 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
                 c_lo = c_hi;
                 __syncthreads();
             }
-        } else if (d > 3 && M > 0) {
+        } else if (d > 3 && M > 0 && !ball) {
             // landmark filter, then the label scans of the undecided ones
             listed = true;
             for (int c = tid; c < M; c += NT) list[c] = (uint32_t)c;

@@ -32,8 +32,8 @@
 //   3. Otherwise: landmark filter (Section "Landmark-Based Filtering"),
 //      when the build has landmark distances: a candidate h with
 //      sd(u,l) + sd(l,h) < d for a landmark l is pruned at once, one with
-//      |sd(u,l) - sd(l,h)| >= d survives at once; the others are compacted
-//      and go on. Prune (rule 2) for every remaining candidate h. A common
+//      |sd(u,l) - sd(l,h)| >= d survives at once; the others
+//      go on. Prune (rule 2) for every remaining candidate h. A common
 //      hub x of L_<d(u) and L_<d(h) with d_u(x) + d_h(x) < d exists iff
 //      some x in L_k(h), 1 <= k <= d-2, has d_u(x) <= d-1-k (the case
 //      k = 0, x = h, was handled in step 2; entries of h at distance d-1
@@ -42,7 +42,10 @@
 //      order with early exit: 8 lanes level by level when u has many
 //      candidates; 16 or 32 lanes over G levels' descriptors read at once,
 //      scanned as one list, when it has few (deep levels of high-diameter
-//      graphs), so that their lanes stay busy.
+//      graphs), so that their lanes stay busy; from kDeferLevel on they are
+//      queued for k_scan_deferred.
+//      At a level that has a distance ball (pspc_ball.cu) one bit of u's row
+//      stands for step 1, the membership test and all of rule 2.
 //   4. Survivors are put in hub order (the rank of a hub is a popcount over
 //      a bitmap of the survivors, or a bitonic sort when that bitmap does
 //      not fit) and appended to the label arena as L_d(u); the arena slot
@@ -316,6 +319,12 @@ struct HashMap {
 // only be at distance d-2-k or d-1-k from u (triangle inequality with
 // sd(u,h) >= d-2). So two binary searches in u's hub-sorted level segments
 // answer every test, and nothing is built per vertex.
+// u's row of the ball, and whether it holds id x (cbase: first id of u's graph).
+__device__ __forceinline__ const uint32_t* ball_of(const LevelArgs& A, int64_t u) {
+    return A.ball ? A.ball + (A.ball_rows.off ? __ldg(A.ball_rows.off + u) : u * A.ball_rows.words) : nullptr;
+}
+__device__ __forceinline__ bool in_ball(const uint32_t* row, uint32_t r) { return (__ldg(row + (r >> 5)) >> (r & 31)) & 1u; }
+
 struct SegMap {
     const uint64_t* seg;
     const uint32_t* hub_arena;
@@ -1089,7 +1098,8 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         __syncthreads();
 
         // 1. label map of L_<d(u)
-        for (int l = 0; l < d && kMap != kMapSeg; ++l) {
+        const uint32_t* ball = ball_of(A, u);  // with a ball the maps are not needed
+        for (int l = 0; l < d && kMap != kMapSeg && !ball; ++l) {
             const uint64_t s = __ldg(A.seg + (int64_t)l * n + u);
             const uint32_t len = seg_len(s);
             const uint32_t* hs = A.hub_arena + seg_start(s);
@@ -1104,7 +1114,7 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         // first ids that the table region can hold (the region is free
         // until the prune step is done). Each thread walks hub-sorted
         // segments, so it stops at the first hub beyond the window.
-        if (kMap == kMapSeg && d > 1) {
+        if (kMap == kMapSeg && d > 1 && !ball) {
             uint32_t cw = (uint32_t)((L.list - L.map) / 4) / (uint32_t)(d - 1);
             cw = cw < kSegCacheMaxWords ? cw : kSegCacheMaxWords;
             if (cw >= kSegCacheMinWords) {
@@ -1179,7 +1189,8 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
                     for (int t = 0; t < kGatherUnroll; ++t)
                         if (ok[t]) {
                             const uint32_t h = hw[t] & kHubMask;
-                            ok[t] = !(kMap == kMapBitmap ? bm.member(h) : kMap == kMapHash ? hm.member(h) : sm.member(h));
+                            ok[t] = !(ball ? in_ball(ball, h - cbase)
+                                      : kMap == kMapBitmap ? bm.member(h) : kMap == kMapHash ? hm.member(h) : sm.member(h));
                         }
                     uint64_t cv[kGatherUnroll];
     #pragma unroll
@@ -1240,9 +1251,9 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         // the range (x, u) of x's sorted row; a hub met there that is a
         // candidate (bitmap cand_bm) is marked pruned (bitmap mk). This replaces
         // scanning L_1(h) for every candidate h.
-        bool marked = false;
+        bool marked = ball != nullptr;  // the ball left survivors only
         const uint32_t Wm = (uint32_t)((u - cbase + 31) >> 5);
-        if (d == 3 && (size_t)Wm * 8 <= (size_t)(L.list - L.map) && M > 0) {
+        if (d == 3 && !marked && (size_t)Wm * 8 <= (size_t)(L.list - L.map) && M > 0) {
             uint32_t* cand_bm = (uint32_t*)mapr;
             uint32_t* mk = cand_bm + Wm;
             for (uint32_t i = tid; i < 2 * Wm; i += NT) cand_bm[i] = 0u;
@@ -1585,7 +1596,7 @@ __device__ void micro_merge(const LevelArgs& A, Mem& m, int T, int64_t u, int64_
     int n_open = 0;
     unsigned int q0 = 0;  // their places in the queue of deferred scans
     bool defer = false;
-    if (d >= 3 && uniq > 0) {
+    if (d >= 3 && uniq > 0 && !A.ball) {
         if (A.lmk) {
             __syncwarp();
             for (int i = lane; i < A.lmk_stride / 4; i += 32)
@@ -1719,7 +1730,9 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
         const uint64_t own1 = __ldg(seg_prev + u);
         const uint64_t own2 = d > 2 ? __ldg(A.seg + (int64_t)(d - 2) * n + u) : 0ull;
         const uint32_t n1 = seg_len(own1), n2 = seg_len(own2);
-        const bool staged = n1 + n2 <= (uint32_t)kMicroOwn;
+        const uint32_t* ball = ball_of(A, u);  // answers for the segments, and for rule 2
+        const uint32_t cbase = ball && A.comp_base ? (uint32_t)__ldg(A.comp_base + u) : 0u;
+        const bool staged = !ball && n1 + n2 <= (uint32_t)kMicroOwn;
         if (staged)
             for (uint32_t i = lane; i < n1 + n2; i += 32)
                 m.u.own[i] = __ldg(A.hub_arena + (i < n1 ? seg_start(own1) : seg_start(own2) - n1) + i) & kHubMask;
@@ -1733,6 +1746,7 @@ __global__ void __launch_bounds__(kMicroThreads) k_level_micro(const LevelArgs A
             return lo < len && xs[lo] == x;
         };
         auto member = [&](uint32_t x) {
+            if (ball) return in_ball(ball, x - cbase);
             if (staged) return find(m.u.own, n1, x) || find(m.u.own + n1, n2, x);
             const uint32_t* h1 = A.hub_arena + seg_start(own1);
             const uint32_t* h2 = A.hub_arena + seg_start(own2);

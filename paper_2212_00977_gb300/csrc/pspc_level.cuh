@@ -117,6 +117,21 @@ struct DeferredScan {
     int32_t pos;   // which of its entries
 };
 
+// Rows of a distance ball (pspc_ball.cu): row u starts at word off[u] (n + 1
+// values; batches), or at u * words. A multiple of 4 words each; bit r is the
+// vertex r after the first of u's graph.
+struct BallRows {
+    const int64_t* off;
+    int64_t words;
+};
+constexpr int64_t kBallBytes = (int64_t)1 << 31;  // most bytes of one ball (two are held)
+// slices: arcs / 128 + 1 pairs. total_words: of one ball; max_words: of its longest row.
+cudaError_t launch_ball_init(int64_t n, int64_t arcs, const int64_t* rp, const int32_t* arc_src, const int32_t* col,
+                             const int32_t* comp_base, const BallRows& R, int64_t total_words, uint32_t* ball, int2* slices,
+                             int* n_slices, cudaStream_t st);
+cudaError_t launch_ball_step(int64_t n, const int64_t* rp, const int32_t* col, const BallRows& R, int64_t max_words,
+                             const int2* slices, int n_slices, const uint32_t* from, uint32_t* to, cudaStream_t st);
+
 struct LevelArgs {
     int d;
     int64_t n;
@@ -154,6 +169,8 @@ struct LevelArgs {
     const uint8_t* lmk;   // [n][lmk_stride] bytes of uint16 landmark distances, or NULL (no filter)
     int lmk_stride;       // bytes per row: a multiple of 16, <= 2 kLmkMax
     int lmk_words;        // 16-byte words of each row the filter tests at this level
+    const uint32_t* ball; // ball d-1 (rule 2 is a bit of it), or NULL
+    BallRows ball_rows;
     HeldSegment* held;    // deferred scans (NULL: scans run in place)
     DeferredScan* scans;
     unsigned int scan_cap;
