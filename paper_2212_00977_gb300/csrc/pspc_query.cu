@@ -799,17 +799,27 @@ constexpr uint32_t kBySourceCand = 256;
 
 // Adds the count products of the warp's list to the lanes' partial sums:
 // lane i takes entries i, i + 32, ..., so the loads are independent.
-template <bool kWords>
+// kByHub: the entries hold the hub instead, whose position is searched in the
+// run's hubs on chip (hubs[0..la)).
+template <bool kWords, bool kByHub>
 __device__ __forceinline__ void add_candidates(const QueryArgs& Q, int64_t a0, const unsigned long long* cntt,
-                                               const uint16_t* distt, const uint32_t* cw, uint32_t nc, int lane, uint64_t& sum,
+                                               const uint16_t* distt, const uint16_t* hubs, uint32_t la, const uint32_t* cw, uint32_t nc, int lane, uint64_t& sum,
                                                uint32_t& flag) {
     __syncwarp();
     for (uint32_t c = lane; c < nc; c += 32) {
         const uint32_t v = cw[c];
-        const uint64_t ca = __ldg((const unsigned long long*)Q.cnt + a0 + ((v >> 1) & 0x7FFFu));
+        uint32_t ia = (v >> 1) & 0x7FFFu;
+        if (kByHub) {
+            uint32_t lo = 0, hi = la;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (hubs[mid] < (v & 0xFFFFu)) lo = mid + 1; else hi = mid;
+            }
+            ia = lo;
+        }
+        const uint64_t ca = __ldg((const unsigned long long*)Q.cnt + a0 + ia);
         const uint64_t cb = __ldg(cntt + (v >> 16));
-        const uint32_t f = kWords ? (uint32_t)(__ldg(Q.dist + a0 + ((v >> 1) & 0x7FFFu)) | __ldg(distt + (v >> 16))) >> 15
-                                  : v & 1u;
+        const uint32_t f = kWords ? (uint32_t)(__ldg(Q.dist + a0 + ia) | __ldg(distt + (v >> 16))) >> 15 : v & 1u;
         add_term(sum, flag, ca * cb, f | (uint32_t)(__umul64hi(ca, cb) != 0));
     }
     __syncwarp();
@@ -835,7 +845,13 @@ __device__ __forceinline__ void add_candidates(const QueryArgs& Q, int64_t a0, c
 // sector each and one load round trip each inside the stream. On an index
 // with words the stream is the words alone, and the flags are read with the
 // counts.
-template <bool kWords>
+//
+// kByHub (words, at most 65,536 vertices): pos[h] holds the distance of hub h
+// itself and sd[i] the hub of entry i, so an entry of L(t) costs one shared
+// read instead of two dependent ones, and positions are searched for the few
+// matches that are kept (10^7 pairs on R-MAT 65,536 16.5 -> 15.3 ms; deep
+// indexes keep many matches: grid 256x256 172 -> 201 ms with it).
+template <bool kWords, bool kByHub>
 __global__ void __launch_bounds__(kBySourceThreads)
     k_query_by_source_direct(const QueryArgs Q, uint32_t n_pad, uint32_t label_pad) {
     extern __shared__ uint16_t dsm[];
@@ -876,8 +892,10 @@ __global__ void __launch_bounds__(kBySourceThreads)
             const uint32_t la = (uint32_t)(__ldg(Q.off + rs + 1) - a0);
             for (uint32_t i = tid; i < la; i += blockDim.x) {
                 const uint32_t w = (uint32_t)__ldg(Q.hub + a0 + i);
-                pos[kWords ? w >> Q.sh : w] = (uint16_t)i;
-                sd[i] = kWords ? (uint16_t)(w >> Q.cb & dmask) : __ldg(Q.dist + a0 + i);
+                const uint32_t h = kWords ? w >> Q.sh : w;
+                const uint16_t da = kWords ? (uint16_t)(w >> Q.cb & dmask) : __ldg(Q.dist + a0 + i);
+                pos[h] = kByHub ? (uint16_t)(da & 0x7FFFu) : (uint16_t)i;
+                sd[i] = kByHub ? (uint16_t)h : da;
             }
             if (tid == 0) s_next = (unsigned long long)r0;
             __syncthreads();
@@ -929,15 +947,17 @@ __global__ void __launch_bounds__(kBySourceThreads)
                     for (int u = 0; u < kBySourceUnroll; ++u) {
                         const uint32_t ia = hb[u] == kNoHub ? 0xFFFFu : (uint32_t)pos[kWords ? hb[u] >> Q.sh : hb[u]];
                         if (kWords) db[u] = hb[u] >> Q.cb & dmask;
-                        const uint32_t da = ia == 0xFFFFu ? 0u : (uint32_t)sd[ia];
-                        key[u] = ia == 0xFFFFu ? 0xFFFFFFFFu
-                                               : ((da & 0x7FFFu) + (db[u] & 0x7FFFu)) << 16 | ia << 1 | ((da | db[u]) >> 15);
+                        if (kByHub) {
+                            key[u] = ia == 0xFFFFu ? 0xFFFFFFFFu : (ia + (db[u] & 0x7FFFu)) << 16 | (hb[u] >> (kWords ? Q.sh : 0));
+                        } else {
+                            const uint32_t da = ia == 0xFFFFu ? 0u : (uint32_t)sd[ia];
+                            key[u] = ia == 0xFFFFu ? 0xFFFFFFFFu
+                                                   : ((da & 0x7FFFu) + (db[u] & 0x7FFFu)) << 16 | ia << 1 | ((da | db[u]) >> 15);
+                        }
                         kmin = min(kmin, key[u]);
                     }
                     // the matches at the running minimum join the warp's list
-                    uint32_t cmin = kmin >> 16;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) cmin = min(cmin, __shfl_xor_sync(0xFFFFFFFFu, cmin, o));
+                    const uint32_t cmin = __reduce_min_sync(0xFFFFFFFFu, kmin) >> 16;
                     if (cmin == 0xFFFFu || cmin > best) continue;  // warp-uniform
                     if (cmin < best) {  // a smaller sum: what the list and the sum hold is superseded
                         best = cmin;
@@ -951,7 +971,7 @@ __global__ void __launch_bounds__(kBySourceThreads)
                         const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
                         if (m == 0) continue;
                         if (nc + (uint32_t)__popc(m) > kBySourceCand) {  // rare: a full list
-                            add_candidates<kWords>(Q, a0, cntt, distt, cw, nc, lane, sum, flag);
+                            add_candidates<kWords, kByHub>(Q, a0, cntt, distt, sd, la, cw, nc, lane, sum, flag);
                             nc = 0;
                         }
                         if (hit)
@@ -960,7 +980,7 @@ __global__ void __launch_bounds__(kBySourceThreads)
                         nc += (uint32_t)__popc(m);
                     }
                 }
-                add_candidates<kWords>(Q, a0, cntt, distt, cw, nc, lane, sum, flag);
+                add_candidates<kWords, kByHub>(Q, a0, cntt, distt, sd, la, cw, nc, lane, sum, flag);
                 finish_pair_warp(Q, p, best == 0xFFFFu ? 0xFFFFFFFFu : best, sum, flag, lane);
             }
             __syncthreads();
@@ -1006,6 +1026,14 @@ constexpr uint32_t kBySourceMaxSlots = 16384;  // 128 KB of table
 // the kernel's static arrays).
 constexpr size_t kBySourceDirectBytes = 224 * 1024;
 
+// The position-table kernel for an index without words, or with them and of
+// at most 65,536 vertices (by_hub) or more.
+static const void* direct_kernel(bool words, bool by_hub) {
+    return !words   ? (const void*)k_query_by_source_direct<false, false>
+           : by_hub ? (const void*)k_query_by_source_direct<true, true>
+                    : (const void*)k_query_by_source_direct<true, false>;
+}
+
 static void set_query_carveouts() {
     std::call_once(g_carveout_once, [] {
         prefer_max_shared((const void*)k_query_by_source);
@@ -1015,7 +1043,7 @@ static void set_query_carveouts() {
             prefer_max_shared(f);
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordBytes);
         }
-        for (const void* f : {(const void*)k_query_by_source_direct<false>, (const void*)k_query_by_source_direct<true>}) {
+        for (const void* f : {direct_kernel(false, false), direct_kernel(true, false), direct_kernel(true, true)}) {
             prefer_max_shared(f);
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBySourceDirectBytes);
         }
@@ -1132,19 +1160,26 @@ static cudaError_t launch_query(Index& ix, const QueryArgs& Q, cudaStream_t st) 
         return cudaGetLastError();
     }
     if (G == PSPC_QUERY_BY_SOURCE && by_source_direct_bytes(ix) > 0) {
-        // positions above a ninth of the shared memory leave room for one CTA
-        // per SM: make it a large one; smaller tables share SMs
+        // as small as leaves an SM 32 warps: a run of pairs ends at a barrier,
+        // and smaller CTAs wait for fewer warps there (2x10^6 pairs: on grid
+        // 128x128 10.2 ms with one CTA of 1,024 threads, 9.9 with four of 256; on
+        // BA 20,011 3.15 and 2.75)
         const size_t base = by_source_direct_bytes(ix);
-        const int threads = base > (size_t)24 * 1024 ? kBySourceThreads : kQueryThreads;
+        auto fits = [&](int threads) {
+            return (base + (size_t)(threads / 32) * kBySourceCand * 4 + 1024) * (1024 / threads) <= kBySourceDirectBytes;
+        };
+        const int threads = fits(256) ? 256 : fits(512) ? 512 : kBySourceThreads;
         const size_t smem = base + (size_t)(threads / 32) * kBySourceCand * 4;
-        const void* f = ix.db ? (const void*)k_query_by_source_direct<true> : (const void*)k_query_by_source_direct<false>;
+        const bool by_hub = ix.db != 0 && ix.n <= 65536;
+        const void* f = direct_kernel(ix.db != 0, by_hub);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, threads, smem);
         if (e != cudaSuccess) return e;
         const int64_t items = (Q.q + kBySourceItem - 1) / kBySourceItem;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, (int64_t)sms * std::max(occ, 1)));
         const uint32_t n_pad = (uint32_t)((ix.n + 1) & ~(int64_t)1), l_pad = by_source_label_pad(ix);
-        if (ix.db) k_query_by_source_direct<true><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
-        else k_query_by_source_direct<false><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
+        if (by_hub) k_query_by_source_direct<true, true><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
+        else if (ix.db) k_query_by_source_direct<true, false><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
+        else k_query_by_source_direct<false, false><<<grid, threads, smem, st>>>(Q, n_pad, l_pad);
         return cudaGetLastError();
     }
     if (G == PSPC_QUERY_BY_SOURCE || G == PSPC_QUERY_BY_SOURCE_HASH) {
