@@ -621,6 +621,7 @@ static void dfree(T*& p, cudaStream_t st) {
 
 struct LevelPlan {
     int map_kind = kMapBitmap;
+    int asked_kind = -1;  // map kind that `occupancy` is for
     uint32_t cap_c = 0, cap_u = 0, bm_words = 0;
     int64_t label_limit = 0;
     size_t smem_bytes = 0;
@@ -696,7 +697,7 @@ struct Builder {
     size_t gscratch_bytes = 0;
     std::vector<unsigned long long> lvl_base;
     Index out;
-    cudaEvent_t ek0 = nullptr, ek1 = nullptr;
+    cudaEvent_t ek0 = nullptr, ek1 = nullptr, ev_level = nullptr;
     float kernel_ms = 0.f;  // level-kernel time of the current level
     float offchip_ms = 0.f; // of which the off-chip variant
     int smem_optin = 0;
@@ -745,7 +746,10 @@ struct Builder {
         cudaStreamSynchronize(st);
     }
 
+    // The status as of now; ends the level's time (ev_level) here, so that no
+    // other wait is needed for it.
     int read_status() {
+        if (ev_level) cudaEventRecord(ev_level, st);
         PSPC_TRY_CUDA(cudaMemcpyAsync(hstt, stt, sizeof(LevelStatus), cudaMemcpyDeviceToHost, st));
         PSPC_TRY_CUDA(cudaStreamSynchronize(st));
         return PSPC_OK;
@@ -1246,12 +1250,19 @@ struct Builder {
             plan.map_kind = kMapSeg;
             plan.label_limit = INT64_MAX;
         }
-        plan.smem_bytes = level_layout(plan.cap_c, level_map_bytes(plan.map_kind, d, plan.bm_words, plan.cap_u)).total;
-        if (plan.smem_bytes + 1024 > (size_t)smem_optin) return PSPC_E_INVAL;  // tables must fit on chip
-        PSPC_TRY_CUDA(level_kernel_attrs(plan.map_kind, plan.smem_bytes, &plan.occupancy));
+        const size_t bytes = level_layout(plan.cap_c, level_map_bytes(plan.map_kind, d, plan.bm_words, plan.cap_u)).total;
+        if (bytes + 1024 > (size_t)smem_optin) return PSPC_E_INVAL;  // tables must fit on chip
+        // the runtime is asked once for each shape (the deep levels share one)
+        if (plan.occupancy == 0 || bytes != plan.smem_bytes || plan.map_kind != plan.asked_kind) {
+            PSPC_TRY_CUDA(level_kernel_attrs(plan.map_kind, bytes, &plan.occupancy));
+            plan.smem_bytes = bytes;
+            plan.asked_kind = plan.map_kind;
+        }
         if (plan.occupancy < 1) return PSPC_E_INVAL;
-        plan.light_smem_bytes = level_layout(kLightCap, level_map_bytes(kMapSeg, d, 0, 0), kLightThreads).total;
-        PSPC_TRY_CUDA(level_kernel_attrs(kMapSeg, plan.light_smem_bytes, &plan.light_occupancy, kLightThreads));
+        if (plan.light_occupancy == 0) {  // the same for every level
+            plan.light_smem_bytes = level_layout(kLightCap, level_map_bytes(kMapSeg, d, 0, 0), kLightThreads).total;
+            PSPC_TRY_CUDA(level_kernel_attrs(kMapSeg, plan.light_smem_bytes, &plan.light_occupancy, kLightThreads));
+        }
         if (plan.light_occupancy < 1) return PSPC_E_INVAL;
         if (plan.micro_occupancy == 0) {  // the same for every level
             PSPC_TRY_CUDA(micro_kernel_occupancy(4, &plan.micro_occupancy));
@@ -1419,6 +1430,7 @@ struct Builder {
         PSPC_TRY_CUDA(cudaEventCreate(&e1));
         PSPC_TRY_CUDA(cudaEventCreate(&ek0));
         PSPC_TRY_CUDA(cudaEventCreate(&ek1));
+        ev_level = e1;
         int levels = 1;
         // Distances are stored in 15 bits: a level beyond the limit that
         // adds an entry ends the build with PSPC_E_DIST (one that adds
@@ -1448,15 +1460,13 @@ struct Builder {
                 levels = 2;
                 continue;
             }
-            cudaMemsetAsync(seg + (int64_t)d * n, 0, n * 8, st);
-            cudaMemsetAsync(stt, 0, sizeof(LevelStatus), st);
-            cudaMemcpyAsync(&stt->bump, &lvl_base[d], 8, cudaMemcpyHostToDevice, st);
+            cudaError_t ce = launch_level_begin(n, seg + (int64_t)d * n, raw_u, stt, lvl_base[d], st);
+            out.launches += 1;
             // Dense-prefix skip on the shallow levels (the prefix pass reads
             // d segments per vertex; deep levels of high-diameter graphs gain
             // little from it).
             skip_prefix = d >= 3 && d <= kDensePrefixMaxLevel && prefix_pays;
-            cudaError_t ce = cudaSuccess;
-            if (skip_prefix) {
+            if (ce == cudaSuccess && skip_prefix) {
                 ce = launch_dense_prefix(d, n, seg, hub_arena, comp_base, hpre, st);
                 out.launches += 1;
             }
@@ -1525,11 +1535,9 @@ struct Builder {
                 *hstt = keep;
             }
             if (rc) break;
-            cudaEventRecord(e1, st);
             bump = hstt->bump;
             const long long added = (long long)(bump - lvl_base[d] - hstt->dropped);
             float ms = 0.f;
-            cudaEventSynchronize(e1);
             cudaEventElapsedTime(&ms, e0, e1);
             pspc_level_stat_t ls{};
             ls.raw_candidates = raw_total + (long long)hstt->prefix_skipped;
@@ -1561,6 +1569,7 @@ struct Builder {
             lvl_base.push_back(bump);
             levels = d + 1;
         }
+        ev_level = nullptr;
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         if (rc) return rc;

@@ -274,7 +274,9 @@ constexpr int kDensePrefixMaxLevel = 8;  // deeper levels: no skip (cost grows w
 constexpr double kDensePrefixMinGain = 0.10;  // stop skipping once it saves less than this share of a level's pulls
 cudaError_t launch_dense_prefix(int d, int64_t n, const uint64_t* seg, const uint32_t* hub_arena,
                                 const int32_t* comp_base, int32_t* hpre, cudaStream_t st);
-// hpre NULL: no skip (arc_lo is not written).
+cudaError_t launch_level_begin(int64_t n, uint64_t* seg_row, int64_t* raw_u, LevelStatus* stt, unsigned long long bump,
+                               cudaStream_t st);
+// hpre NULL: no skip (arc_lo is not written). raw_u has to be zero.
 cudaError_t launch_cost(int d, int64_t n, int64_t arcs, const int64_t* rp, const int32_t* col,
                         const int32_t* arc_src, const uint64_t* seg_prev, const uint32_t* hub_arena,
                         const int32_t* hpre, uint32_t* arc_lo, uint32_t* cnt_arc, int64_t* raw_u,
