@@ -1291,7 +1291,7 @@ struct Builder {
         PSPC_TRY_CUDA(cudaEventCreate(&a));
         PSPC_TRY_CUDA(cudaEventCreate(&b));
         cudaEventRecord(a, st);
-        int rc = landmark_bfs(n, rp_r, col_r, comp_base, out.lmk_k, out.lmk_stride, out.lmk, out.lmk_ids, st,
+        int rc = landmark_bfs(n, arcs, rp_r, col_r, comp_base, out.lmk_k, out.lmk_stride, out.lmk, out.lmk_ids, st,
                               &out.launches);
         cudaEventRecord(b, st);
         if (!rc) {

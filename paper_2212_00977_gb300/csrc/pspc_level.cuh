@@ -250,7 +250,7 @@ __host__ __device__ inline size_t level_map_bytes(int kind, int d, uint32_t bm_w
 // row, 0xFFFF where the distance is undefined (unreached, or no such
 // landmark). ids (NULL, or host int32[64] out): the id of landmark j, -1 for
 // none. Synchronises st every few BFS levels.
-int landmark_bfs(int64_t n, const int64_t* rp, const int32_t* col, const int32_t* comp_base, int k, int stride,
+int landmark_bfs(int64_t n, int64_t arcs, const int64_t* rp, const int32_t* col, const int32_t* comp_base, int k, int stride,
                  uint8_t* ld, int32_t* ids, cudaStream_t st, int64_t* launches);
 
 // Push paradigm (Algorithm PUSH): every arc u->v sends u the entries of
