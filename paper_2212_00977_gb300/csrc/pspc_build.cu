@@ -689,7 +689,9 @@ struct Builder {
     DeferredScan* scans = nullptr;   // (and behind it the scans left after the proof)
     unsigned int scan_cap = 0;
     int32_t* glist = nullptr;
-    LevelStatus* stt = nullptr;
+    LevelStatus* stt = nullptr;     // the level's of two_stt, in turn
+    LevelStatus* two_stt = nullptr;
+    int max_deg = -1;               // known from level 2 on
     LevelStatus hs;               // host copy of the level status
     LevelStatus* hstt = &hs;
     int* err = nullptr;
@@ -731,7 +733,7 @@ struct Builder {
         dfree(held, st);
         dfree(scans, st);
         dfree(glist, st);
-        dfree(stt, st);
+        dfree(two_stt, st);
         dfree(err, st);
         dfree(gscratch, st);
         if (ek0) cudaEventDestroy(ek0);
@@ -1413,7 +1415,7 @@ struct Builder {
         PSPC_TRY_CUDA(dalloc(&lab_size, n, st));
         PSPC_TRY_CUDA(dalloc(&items, n, st));
         PSPC_TRY_CUDA(dalloc(&glist, 2 * n, st));
-        PSPC_TRY_CUDA(dalloc(&stt, 1, st));
+        PSPC_TRY_CUDA(dalloc(&two_stt, 2, st));
         PSPC_TRY_CUDA(cudaMemsetAsync(lab_size, 0, n * 8, st));
         PSPC_TRY_CUDA(launch_arc_src(rp_r, n, arc_src, st));
         out.launches += 1;
@@ -1460,8 +1462,14 @@ struct Builder {
                 levels = 2;
                 continue;
             }
-            cudaError_t ce = launch_level_begin(n, seg + (int64_t)d * n, raw_u, stt, lvl_base[d], st);
-            out.launches += 1;
+            stt = two_stt + d % 2;
+            LevelStatus* next = two_stt + (d + 1) % 2;
+            const bool small_degrees = max_deg >= 0 && max_deg <= kCostMaxDegree;
+            cudaError_t ce = cudaSuccess;
+            if (!small_degrees) {
+                ce = launch_level_begin(n, seg + (int64_t)d * n, raw_u, stt, next, lvl_base[d], st);
+                out.launches += 1;
+            }
             // Dense-prefix skip on the shallow levels (the prefix pass reads
             // d segments per vertex; deep levels of high-diameter graphs gain
             // little from it).
@@ -1473,12 +1481,20 @@ struct Builder {
             // the largest count of level d-1 (level 1: every count is 1)
             const DenseRule dense{plan.dense_occupancy > 0, d == 2 ? 1u : hstt->cmax,
                                   o.granular ? kDenseMinRawGranular : kDenseMinRaw, comp_base};
-            if (ce == cudaSuccess)
-                ce = launch_cost(d, n, arcs, rp_r, col_r, arc_src, seg + (int64_t)(d - 1) * n, hub_arena,
-                                 skip_prefix ? hpre : nullptr, arc_lo, cnt_arc, raw_u, lab_size, stt,
-                                 plan.label_limit, dense, glist, items, st, &out.launches);
+            const int32_t* prefix = skip_prefix ? hpre : nullptr;
+            if (ce == cudaSuccess && small_degrees) {
+                ce = launch_cost_level(n, rp_r, col_r, seg + (int64_t)(d - 1) * n, seg + (int64_t)d * n, hub_arena, prefix,
+                                       arc_lo, cnt_arc, raw_u, lab_size, stt, next, lvl_base[d], plan.label_limit, dense,
+                                       glist, items, st);
+                out.launches += 2;
+            } else if (ce == cudaSuccess) {
+                ce = launch_cost(d, n, arcs, rp_r, col_r, arc_src, seg + (int64_t)(d - 1) * n, hub_arena, prefix, arc_lo,
+                                 cnt_arc, raw_u, lab_size, stt, plan.label_limit, dense, glist, items,
+                                 max_deg < 0 ? &stt->max_deg : nullptr, st, &out.launches);
+            }
             if ((rc = cuda_status(ce))) break;
             if ((rc = read_status())) break;
+            if (max_deg < 0) max_deg = hstt->max_deg;
             if (hstt->n_active == 0) break;
             const long long raw_total = (long long)hstt->raw_total;
             // Push paradigm: the arcs send their entries into per-vertex

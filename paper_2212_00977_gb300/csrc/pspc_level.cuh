@@ -83,6 +83,7 @@ struct LevelStatus {
     unsigned int n_scan_open;    // of them, left after the neighbours' proof
     unsigned int n_scan;         // deferred scans asked for (those past the queue's size run in place)
     unsigned long long dropped;  // entries that deferred scans took out of their segments
+    int max_deg;     // largest degree of the graph (level 2 only)
     int work_dense;
     unsigned int cmax;  // largest count appended at this level (0xFFFFFFFF: 2^32 or more, or flagged)
     // on-chip attempts and overflows of vertices that can overflow, by
@@ -274,14 +275,24 @@ constexpr int kDensePrefixMaxLevel = 8;  // deeper levels: no skip (cost grows w
 constexpr double kDensePrefixMinGain = 0.10;  // stop skipping once it saves less than this share of a level's pulls
 cudaError_t launch_dense_prefix(int d, int64_t n, const uint64_t* seg, const uint32_t* hub_arena,
                                 const int32_t* comp_base, int32_t* hpre, cudaStream_t st);
-cudaError_t launch_level_begin(int64_t n, uint64_t* seg_row, int64_t* raw_u, LevelStatus* stt, unsigned long long bump,
-                               cudaStream_t st);
-// hpre NULL: no skip (arc_lo is not written). raw_u has to be zero.
+cudaError_t launch_level_begin(int64_t n, uint64_t* seg_row, int64_t* raw_u, LevelStatus* stt, LevelStatus* next,
+                               unsigned long long bump, cudaStream_t st);
+// hpre NULL: no skip (arc_lo is not written). raw_u has to be zero. max_deg
+// (may be NULL): the largest degree, for what is there already.
 cudaError_t launch_cost(int d, int64_t n, int64_t arcs, const int64_t* rp, const int32_t* col,
                         const int32_t* arc_src, const uint64_t* seg_prev, const uint32_t* hub_arena,
                         const int32_t* hpre, uint32_t* arc_lo, uint32_t* cnt_arc, int64_t* raw_u,
                         int64_t* lab_size, LevelStatus* stt, int64_t label_limit, const DenseRule& dense,
-                        int32_t* glist, int32_t* items, cudaStream_t st, int64_t* launches);
+                        int32_t* glist, int32_t* items, int* max_deg, cudaStream_t st, int64_t* launches);
+// launch_level_begin and launch_cost in two launches, for graphs of degrees
+// up to kCostMaxDegree: four lanes walk the arcs of a vertex there. *stt was
+// cleared as the `next` of the level before.
+constexpr int kCostMaxDegree = 32;
+cudaError_t launch_cost_level(int64_t n, const int64_t* rp, const int32_t* col, const uint64_t* seg_prev,
+                              uint64_t* seg_row, const uint32_t* hub_arena, const int32_t* hpre, uint32_t* arc_lo,
+                              uint32_t* cnt_arc, int64_t* raw_u, int64_t* lab_size, LevelStatus* stt, LevelStatus* next,
+                              unsigned long long bump, int64_t label_limit, const DenseRule& dense, int32_t* glist,
+                              int32_t* items, cudaStream_t st);
 cudaError_t level_kernel_attrs(int map_kind, size_t smem_bytes, int* occupancy, int nt = kLevelThreads);
 cudaError_t launch_level(int map_kind, bool offchip, int grid, size_t smem_bytes, const LevelArgs& A,
                          cudaStream_t st, int nt = kLevelThreads);
