@@ -1065,11 +1065,19 @@ struct Builder {
         // shallow levels test the first kLmkShallow landmarks only: their
         // short distances seldom prove survival, and half the row is read
         A.lmk_words = d < kLmkDeepLevel ? std::min(out.lmk_stride / 16, 2 * kLmkShallow / 16) : out.lmk_stride / 16;
-        if (d >= kDeferLevel && A.lmk && !A.ball && (int64_t)hstt->n_active * d >= kDeferWork) {
+        const bool defer = d >= kDeferLevel ? (int64_t)hstt->n_active * d >= kDeferWork
+                                            : d >= kDeferShallow && hstt->raw_total >= kDeferPulled;
+        if (defer && A.lmk && !A.ball) {
             if (!held) {
                 scan_cap = (unsigned)std::min<int64_t>(std::max<int64_t>(4 * n, 1 << 16), 1 << 26);
-                PSPC_TRY_CUDA(dalloc(&held, n, st));
-                PSPC_TRY_CUDA(dalloc(&scans, 2 * (size_t)scan_cap, st));
+                cudaError_t e = dalloc(&held, n, st);
+                if (e == cudaSuccess) e = dalloc(&scans, 2 * (size_t)scan_cap, st);
+                if (e != cudaSuccess) {  // no room for them: the scans run in place
+                    cudaGetLastError();
+                    dfree(held, st);
+                    held = nullptr;
+                    scans = nullptr;
+                }
             }
             A.held = held;
             A.scans = scans;

@@ -42,7 +42,7 @@
 //      order with early exit: 8 lanes level by level when u has many
 //      candidates; 16 or 32 lanes over G levels' descriptors read at once,
 //      scanned as one list, when it has few (deep levels of high-diameter
-//      graphs), so that their lanes stay busy; from kDeferLevel on they are
+//      graphs), so that their lanes stay busy; in deep or busy levels they are
 //      queued for k_scan_deferred.
 //      At a level that has a distance ball (pspc_ball.cu) one bit of u's row
 //      stands for step 1, the membership test and all of rule 2.
@@ -2182,7 +2182,7 @@ cudaError_t launch_level_micro(int rows, int grid, const LevelArgs& A, cudaStrea
 
 cudaError_t launch_level(int map_kind, bool offchip, int grid, size_t smem_bytes, const LevelArgs& A,
                          cudaStream_t st, int nt) {
-    if (nt == kLightThreads && !offchip && map_kind == kMapSeg && A.d >= kDeferLevel)
+    if (nt == kLightThreads && !offchip && map_kind == kMapSeg && (A.d >= kDeferLevel || A.held))
         k_level<kMapSeg, false, kLightThreads, true><<<grid, nt, smem_bytes, st>>>(A);
     else if (nt == kLightThreads && !offchip) launch_level_nt<kLightThreads>(map_kind, false, grid, smem_bytes, A, st);
     else launch_level_nt<kLevelThreads>(map_kind, offchip, grid, smem_bytes, A, st);

@@ -95,15 +95,21 @@ struct LevelStatus {
     int bucket_fill[kBuckets];
 };
 
-// Deferred label scans of the deep levels. A vertex with undecided
+// Deferred label scans. A vertex with undecided
 // candidates appends them with its survivors and asks for their scans; the
 // scans of all vertices then run evenly over the GPU (k_scan_deferred), and
 // the last one of a vertex closes its segment.
-constexpr int kDeferLevel = 16;  // first level that defers: shorter scans run in place
-// and only with this many active vertices times levels, where the scans are
+constexpr int kDeferLevel = 16;  // from this level on
+// and with this many active vertices times levels, where the scans are
 // worth two launches a level (grid 61x67 builds in 17.2 ms without them, 17.9
 // with 2^17 here; grid 128x128 54 ms either way, grid 256x256 339 and 336).
 constexpr int64_t kDeferWork = 1 << 18;
+// Before it, with this many pulled entries: a vertex with a hundred undecided
+// candidates scans for them one after another while the GPU is idle (R-MAT
+// 65,536, level 5: 788,080 pulled, 2.5 ms in place and 0.4 deferred; of BA
+// 100,000, level 8: 61,290 pulled, 0.18 in place and 0.21 deferred).
+constexpr int kDeferShallow = 4;
+constexpr unsigned long long kDeferPulled = 1 << 18;
 constexpr int kNeighbourLevel = 8;  // from here on a scan costs more than the neighbours' proof that may spare it
 struct HeldSegment {
     unsigned long long start;  // of the entries appended so far in the arena
