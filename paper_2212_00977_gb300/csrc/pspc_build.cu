@@ -1066,7 +1066,8 @@ struct Builder {
         // short distances seldom prove survival, and half the row is read
         A.lmk_words = d < kLmkDeepLevel ? std::min(out.lmk_stride / 16, 2 * kLmkShallow / 16) : out.lmk_stride / 16;
         const bool defer = d >= kDeferLevel ? (int64_t)hstt->n_active * d >= kDeferWork
-                                            : d >= kDeferShallow && hstt->raw_total >= kDeferPulled;
+                                            : d >= kDeferShallow && hstt->raw_total >= kDeferPulled &&
+                                                  hstt->n_active >= kDeferActive;
         if (defer && A.lmk && !A.ball) {
             if (!held) {
                 scan_cap = (unsigned)std::min<int64_t>(std::max<int64_t>(4 * n, 1 << 16), 1 << 26);

@@ -104,12 +104,15 @@ constexpr int kDeferLevel = 16;  // from this level on
 // worth two launches a level (grid 61x67 builds in 17.2 ms without them, 17.9
 // with 2^17 here; grid 128x128 54 ms either way, grid 256x256 339 and 336).
 constexpr int64_t kDeferWork = 1 << 18;
-// Before it, with this many pulled entries: a vertex with a hundred undecided
-// candidates scans for them one after another while the GPU is idle (R-MAT
-// 65,536, level 5: 788,080 pulled, 2.5 ms in place and 0.4 deferred; of BA
-// 100,000, level 8: 61,290 pulled, 0.18 in place and 0.21 deferred).
+// Before it, with this many pulled entries and active vertices: a vertex with
+// a hundred undecided candidates scans for them one after another while the
+// GPU is idle (R-MAT 65,536, level 5: 788,080 pulled, 2.5 ms in place and 0.4
+// deferred). The queue, its allocation and two launches cost some 60 us: of
+// BA 100,000, level 8, 61,290 pulled take 0.18 ms in place and 0.21 deferred,
+// and BA 2,000 builds in 1.04 ms without it, 1.10 with.
 constexpr int kDeferShallow = 4;
 constexpr unsigned long long kDeferPulled = 1 << 18;
+constexpr int kDeferActive = 2048;
 constexpr int kNeighbourLevel = 8;  // from here on a scan costs more than the neighbours' proof that may spare it
 struct HeldSegment {
     unsigned long long start;  // of the entries appended so far in the arena

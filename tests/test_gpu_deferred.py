@@ -47,14 +47,14 @@ def test_odd_cycles(pspc):  # noqa: F811
 
 @pytest.mark.parametrize("n,m", [(2500, 3), (4001, 4)])
 def test_shallow_levels_that_defer(pspc, n, m):  # noqa: F811
-    """Levels 4 to 15 with 2^18 pulled entries or more and no distance ball
-    (which a chosen label map rules out)."""
+    """Levels 4 to 15 with 2^18 pulled entries, 2,048 active vertices or more
+    and no distance ball (which a chosen label map rules out)."""
     g = P.barabasi_albert(n, m, 7)
     rank = P.degree_rank(g, "random", 5)
     ref = oracle.OracleIndex(g, rank).export()
     for kw in (dict(map_kind=1), dict(map_kind=2, landmarks=1), dict(map_kind=3, landmarks=2, warp_levels=15),
                dict(map_kind=1, granular=True)):
         ix = gpu_index(pspc, g, rank, **kw)
-        assert any(l["raw_candidates"] >= 1 << 18 for l in ix.level_stats()[3:])
+        assert any(l["raw_candidates"] >= 1 << 18 and l["active_vertices"] >= 2048 for l in ix.level_stats()[3:])
         assert_index_equal(ix, ref)
         ix.free()
