@@ -43,12 +43,14 @@ constexpr uint32_t kDenseWindow = 11264;    // ids per on-chip window, a multipl
 constexpr uint32_t kDenseBounds = 1024;     // cells of the table of window starts
 constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (32 MB of slab a CTA)
 constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32 + floor(log2 pulled entries)
-// A vertex with fewer pulled entries cannot overflow the on-chip hash and
-// has too few to pay for the windows: R-MAT 2^20 builds in 615 ms with 2,048
-// here, 643 with 3,500, 677 with 5,000 (R-MAT 65,536 12.9, 13.2, 13.4 ms).
-// Per window of its id range it needs 48 more (window overhead against a
-// hash in device memory): 621 ms with 48, 655 with 96, 743 with 1,024.
-constexpr int64_t kDenseMinRaw = 2048;
+// A vertex with fewer pulled entries has too few to pay for the windows; it
+// is one of the light class then. A batch of 96 BA graphs builds in 92 ms with
+// 512 here, 95 with 256, 97 with 768, 102 with 1,024, 109 with 2,048 (R-MAT
+// 262,144 59.0, 59.7, 59.6, 61.2 and 63.7 ms, BA 20,011 3.12, 3.12, 3.21, 3.32
+// and 3.55). Per window of its id range it needs 48 more (window overhead
+// against a hash in device memory): R-MAT 2^20 586 ms with 48, 588 with 64,
+// 616 with 96.
+constexpr int64_t kDenseMinRaw = 512;
 constexpr int64_t kDenseRawPerWindow = 48;
 // Granular builds run one hash CTA per vertex, and the dense kernel at half
 // occupancy: only vertices that would mostly overflow the hash pay (BA

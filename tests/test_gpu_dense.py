@@ -40,6 +40,19 @@ def test_windows_and_rows(pspc, scale, ef, order, kw):
     ix.free()
 
 
+@pytest.mark.parametrize("m", [255, 256, 257])
+def test_fewest_pulled_entries(pspc, m):
+    """Vertices that pull 510, 512 and 514 entries: either side of the line
+    between the hash and the windows."""
+    g = G.hub_ladder(m, 6)
+    rank = np.arange(g.n, dtype=np.int32)
+    ref = oracle.OracleIndex(g, rank).export()
+    for kw in ({}, {"landmarks": -1}, {"max_ctas": 1}):
+        ix = gpu_index(pspc, g, rank, **kw)
+        assert_index_equal(ix, ref)
+        ix.free()
+
+
 @pytest.mark.parametrize("m,depth", [(1500, 34), (1300, 66)])
 def test_counts_up_to_the_bound(pspc, m, depth):
     """Ladder vertices pull 2m entries with counts 2^(level - 1): sums are
