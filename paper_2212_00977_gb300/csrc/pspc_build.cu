@@ -313,17 +313,14 @@ __global__ void k_fin_sizes(int64_t n, int levels, const uint64_t* __restrict__ 
     if ((threadIdx.x & 31) == 0 && m) atomicMax(max_lab, m);
 }
 
-// A word of the finished index (Index::hub); *escapes counts the counts that
-// it cannot hold.
+// A word of the finished index (Index::hub).
 struct WordShape {
     int sh, db, cb;
 };
-__device__ __forceinline__ int32_t hub_word(const WordShape& W, uint32_t h, uint32_t dist, uint64_t cnt, uint32_t ovf,
-                                            unsigned long long* escapes) {
+__device__ __forceinline__ int32_t hub_word(const WordShape& W, uint32_t h, uint32_t dist, uint64_t cnt, uint32_t ovf) {
     if (W.db == 0) return (int32_t)h;
     const uint32_t most = (1u << W.cb) - 1u;
-    const bool escape = ovf != 0 || cnt >= most;
-    *escapes += escape;
+    const bool escape = ovf != 0 || cnt >= most;  // the word cannot hold it
     return (int32_t)(h << W.sh | dist << W.cb | (escape ? most : (uint32_t)cnt));
 }
 
@@ -426,7 +423,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FinArgs F) {
         for (uint32_t i = (uint32_t)T + tid; i < P; i += kFinThreads) keys[i] = ~0ull;
         __syncthreads();
         fin_bitonic_sort(keys, P);
-        unsigned long long novf = 0, nesc = 0;
+        unsigned long long novf = 0;
         for (int64_t i = tid; i < T; i += kFinThreads) {
             const unsigned long long k = keys[i];
             const uint64_t pos = k & ((1ull << 40) - 1);
@@ -438,12 +435,11 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FinArgs F) {
             const uint32_t ovf = __ldg(F.hub_arena + pos) >> 31;
             novf += ovf;
             const uint64_t c = __ldg((const unsigned long long*)F.cnt_arena + pos);
-            F.hub[o0 + i] = hub_word(F.word, (uint32_t)(k >> 40), (uint32_t)lo, c, ovf, &nesc);
+            F.hub[o0 + i] = hub_word(F.word, (uint32_t)(k >> 40), (uint32_t)lo, c, ovf);
             F.dist[o0 + i] = (uint16_t)(lo | (ovf << 15));
             F.cnt[o0 + i] = c;
         }
         if (novf) atomicAdd(&s_ovf, novf);
-        if (nesc) atomicAdd(F.n_ovf + 2, nesc);
         __syncthreads();
     }
     __syncthreads();
@@ -468,7 +464,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize_rank(const FinArgs F) 
     if (tid == 0) s_ovf = 0;
     uint32_t* bits = s_bits;
     uint32_t* wp = s_bits + F.rank_words;
-    unsigned long long novf = 0, nesc = 0;
+    unsigned long long novf = 0;
     for (int64_t u = blockIdx.x; u < F.n; u += gridDim.x) {
         const int64_t o0 = F.off[u];
         const uint32_t cb = F.comp_base ? (uint32_t)__ldg(F.comp_base + u) : 0u;
@@ -512,7 +508,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize_rank(const FinArgs F) 
                         const uint32_t ovf = hw >> 31;
                         novf += ovf;
                         const uint64_t c = __ldg((const unsigned long long*)F.cnt_arena + pos);
-                        F.hub[o0 + rank] = hub_word(F.word, hw & kHubMask, (uint32_t)(l0 + lo), c, ovf, &nesc);
+                        F.hub[o0 + rank] = hub_word(F.word, hw & kHubMask, (uint32_t)(l0 + lo), c, ovf);
                         F.dist[o0 + rank] = (uint16_t)((uint32_t)(l0 + lo) | (ovf << 15));
                         F.cnt[o0 + rank] = c;
                     }
@@ -522,7 +518,6 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize_rank(const FinArgs F) 
         }
     }
     if (novf) atomicAdd(&s_ovf, novf);
-    if (nesc) atomicAdd(F.n_ovf + 2, nesc);
     __syncthreads();
     if (tid == 0 && s_ovf) atomicAdd(F.n_ovf, s_ovf);
 }
@@ -541,7 +536,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize_merge(const FinArgs F)
     const int tid = threadIdx.x;
     const int L = F.levels;
     if (tid == 0) s_ovf = 0;
-    unsigned long long novf = 0, nesc = 0;
+    unsigned long long novf = 0;
     // every vertex, or (F.list) the long labels with a larger on-chip buffer
     const int64_t items = F.list ? (int64_t)F.n_list : F.n;
     for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
@@ -553,7 +548,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize_merge(const FinArgs F)
             if (tid == 0) {
                 const uint64_t s = __ldg(F.seg + u);
                 const uint64_t c = __ldg((const unsigned long long*)F.cnt_arena + seg_start(s));
-                F.hub[o0] = hub_word(F.word, __ldg(F.hub_arena + seg_start(s)) & kHubMask, 0u, c, 0u, &nesc);
+                F.hub[o0] = hub_word(F.word, __ldg(F.hub_arena + seg_start(s)) & kHubMask, 0u, c, 0u);
                 F.dist[o0] = 0;
                 F.cnt[o0] = c;
             }
@@ -594,14 +589,13 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize_merge(const FinArgs F)
             }
             const uint32_t ovf = w >> 31;
             novf += ovf;
-            F.hub[o0 + pos] = hub_word(F.word, h, (uint32_t)l, c, ovf, &nesc);
+            F.hub[o0 + pos] = hub_word(F.word, h, (uint32_t)l, c, ovf);
             F.dist[o0 + pos] = (uint16_t)(l | (ovf << 15));
             F.cnt[o0 + pos] = c;
         }
         __syncthreads();
     }
     if (novf) atomicAdd(&s_ovf, novf);
-    if (nesc) atomicAdd(F.n_ovf + 2, nesc);
     __syncthreads();
     if (tid == 0 && s_ovf) atomicAdd(F.n_ovf, s_ovf);
 }
@@ -1612,9 +1606,9 @@ struct Builder {
         PSPC_TRY_CUDA(dalloc(&big, n, st));
         PSPC_TRY_CUDA(dalloc(&ctr, 2, st));
         PSPC_TRY_CUDA(dalloc(&d_lvl, lvl_base.size(), st));
-        PSPC_TRY_CUDA(dalloc(&n_ovf, 3, st));  // [0] overflow entries, [1] largest label, [2] escapes
+        PSPC_TRY_CUDA(dalloc(&n_ovf, 2, st));  // [0] overflow entries, [1] largest label
         PSPC_TRY_CUDA(cudaMemsetAsync(ctr, 0, 8, st));
-        PSPC_TRY_CUDA(cudaMemsetAsync(n_ovf, 0, 24, st));
+        PSPC_TRY_CUDA(cudaMemsetAsync(n_ovf, 0, 16, st));
         PSPC_TRY_CUDA(cudaMemcpyAsync(d_lvl, lvl_base.data(), lvl_base.size() * 8, cudaMemcpyHostToDevice, st));
         k_fin_sizes<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, L, seg, out.off, big, ctr, n_ovf + 1);
         out.launches += 1;
@@ -1724,11 +1718,10 @@ struct Builder {
             out.launches += 1;
             PSPC_TRY_CUDA(cudaGetLastError());
         }
-        unsigned long long hovf[3] = {0, 0, 0};
-        PSPC_TRY_CUDA(cudaMemcpyAsync(hovf, n_ovf, 24, cudaMemcpyDeviceToHost, st));
+        unsigned long long hovf[2] = {0, 0};
+        PSPC_TRY_CUDA(cudaMemcpyAsync(hovf, n_ovf, 16, cudaMemcpyDeviceToHost, st));
         PSPC_TRY_CUDA(cudaStreamSynchronize(st));
         out.overflow_entries = (int64_t)hovf[0];
-        out.escapes = (int64_t)hovf[2];
         dfree(big, st);
         dfree(ctr, st);
         dfree(d_lvl, st);

@@ -53,7 +53,6 @@ struct Index {
     // where hub and distance do not fit one word.
     int32_t* hub = nullptr;
     int sh = 0, db = 0, cb = 0;
-    int64_t escapes = 0;       // entries whose count is not in their word
     uint16_t* dist = nullptr;  // distance | overflow << 15
     uint64_t* cnt = nullptr;   // trough path count mod 2^64
     int64_t entries = 0;
