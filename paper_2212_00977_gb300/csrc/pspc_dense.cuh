@@ -16,14 +16,16 @@
 // overflow flag) times u's degree is below 2^32. The other vertices keep the
 // hash kernels with 64-bit sums, carries and flags.
 //
-// What bounds it: on R-MAT 2^20, level 3 (3.0e10 pulled entries), half of the
-// CTA cycles are the pull (issue and reads of 12 bytes an entry from L2), a
+// What bounds it: latency. On R-MAT 262,144, level 3, with half the warps it
+// has now, 40% of the issue slots were used, of 20 cycles per issue 8 waited
+// for reads (L2 hits half of the time), 4 at barriers; DRAM was at 12%, L2 at
+// 10%. By phases, on R-MAT 2^20, level 3 (3.0e10 pulled entries): half pull, a
 // fifth the marking walk, a tenth each the member bitmaps and the scans of
 // run lengths; at level 4 the landmark filter and the label scans take 57%.
 // The hash it replaces kept tables of more than 4,096 slots in device memory,
 // half of whose sectors missed L2: levels 3 and 4 took 568 and 495 ms, now
-// 238 and 280 ms (the build 1,182 -> 616 ms; BA 100,000, m = 8: 240 -> 171). With
-// a distance ball its row is the window's bitmap and only the pull is left.
+// 180 and 208 (the build 1,182 -> 488 ms). With a distance ball its row is the
+// window's bitmap and only the pull is left.
 
 // Words of the window's bitmaps.
 constexpr uint32_t kDenseWords = kDenseWindow / 32;

@@ -33,13 +33,15 @@ constexpr int kLmkShallow = 32;    // landmarks the filter tests below level kLm
 constexpr int kLmkDeepLevel = 16;  // from this level on, the filter tests every landmark
 
 // Vertices merged by direct addressing (k_level_dense).
-// Small CTAs: the kernel alternates short phases between barriers, and four
-// CTAs of 256 threads with 11,264-id windows fill each other's gaps better
-// than fewer large ones (R-MAT 2^20 build: 1 x 1024 threads 763 ms, 2 x 512
-// 660 ms, 4 x 256 621 ms, 8 x 128 622 ms but BA 100,000 176 against 171 ms).
+// Small CTAs: the kernel alternates short phases between barriers and waits
+// for its reads (a third of the stalls each), so eight CTAs of 256 threads
+// with 4,608-id windows fill each other's gaps best: R-MAT 2^20 builds in 488
+// ms, with 4 CTAs and 11,264 ids 578, 5 and 8,960 547, 6 and 6,912 505, 7 and
+// 5,760 515, 4 of 512 threads and 10,240 ids 496 (batch of 96 BA graphs 83 ms,
+// 91, 90, 86, 86 and 92).
 constexpr int kDenseThreads = 256;
-constexpr int kDenseBlocks = 4;             // resident CTAs per SM (53 KB of shared memory each)
-constexpr uint32_t kDenseWindow = 11264;    // ids per on-chip window, a multiple of 128
+constexpr int kDenseBlocks = 8;             // resident CTAs per SM (26 KB of shared memory each)
+constexpr uint32_t kDenseWindow = 4608;     // ids per on-chip window, a multiple of 128
 constexpr uint32_t kDenseBounds = 1024;     // cells of the table of window starts
 constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (32 MB of slab a CTA)
 constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32 + floor(log2 pulled entries)
@@ -47,11 +49,11 @@ constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32
 // is one of the light class then. A batch of 96 BA graphs builds in 92 ms with
 // 512 here, 95 with 256, 97 with 768, 102 with 1,024, 109 with 2,048 (R-MAT
 // 262,144 59.0, 59.7, 59.6, 61.2 and 63.7 ms, BA 20,011 3.12, 3.12, 3.21, 3.32
-// and 3.55). Per window of its id range it needs 48 more (window overhead
-// against a hash in device memory): R-MAT 2^20 586 ms with 48, 588 with 64,
-// 616 with 96.
+// and 3.55; all with windows of 11,264 ids). Per window of its id range it
+// needs 12 (window overhead against a hash in device memory): R-MAT 2^20 488
+// ms with 12, 494 with 20.
 constexpr int64_t kDenseMinRaw = 512;
-constexpr int64_t kDenseRawPerWindow = 48;
+constexpr int64_t kDenseRawPerWindow = 12;
 // Granular builds run one hash CTA per vertex, and the dense kernel at half
 // occupancy: only vertices that would mostly overflow the hash pay (BA
 // 20,011: 7.2 ms, with 2,048 here 7.9 ms).
