@@ -702,7 +702,9 @@ __device__ bool scan_filtered(uint32_t* mem, uint32_t words, const uint64_t* __r
                 const uint32_t at = seg_lower_bound(hub_arena + seg_start(s), seg_len(s), x);
                 hit = at < seg_len(s) && (__ldg(hub_arena + seg_start(s) + at) & kHubMask) == x;
             }
-            found = __any_sync(FULL, hit);
+            // a nearly full filter fills the list twice in a row of entries:
+            // the second look-up must not take back what the first one found
+            found |= __any_sync(FULL, hit);
             const uint32_t tail = lane + 32 < nh ? hits[lane + 32] : 0u;
             __syncwarp();
             if (lane + 32 < nh) hits[lane] = tail;
@@ -715,6 +717,7 @@ __device__ bool scan_filtered(uint32_t* mem, uint32_t words, const uint64_t* __r
                 if (b + t * 32 >= nb || found) continue;  // warp-uniform
 #pragma unroll
                 for (int o = 0; o < 2; ++o) {  // x at level l of u: levels d-1-l and d-2-l of h
+                    if (found) continue;  // warp-uniform
                     const int jj = (int)(xb[t] >> 24) - o;
                     bool maybe = false;
                     if (xb[t] != kEmpty && jj >= 0 && jj < 31) {
