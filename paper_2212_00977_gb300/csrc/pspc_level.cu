@@ -1439,10 +1439,10 @@ __global__ void __launch_bounds__(NT, level_min_blocks(NT)) k_level(const LevelA
         unsigned int q0 = 0;
         bool defer = false;
         if (kDeep && A.held && !marked && ns > 0) {
-            if (tid == 0) s_next = (int)atomicAdd(&A.stt->n_scan, (unsigned)ns);
+            if (tid == 0) s_next = (int)scan_place(atomicAdd(&A.stt->n_scan, (unsigned long long)ns), A.scan_cap);
             __syncthreads();
             q0 = (unsigned)s_next;
-            defer = q0 < A.scan_cap && A.scan_cap - q0 >= (unsigned)ns;
+            defer = A.scan_cap - q0 >= (unsigned)ns;
             if (!defer)
                 for (unsigned int i = q0 + tid; i < A.scan_cap && i - q0 < (unsigned)ns; i += NT) A.scans[i].held = -1;
             __syncthreads();
@@ -1736,9 +1736,9 @@ __device__ void micro_merge(const LevelArgs& A, Mem& m, int T, int64_t u, int64_
 #pragma unroll
         for (int j = 0; j < R; ++j) n_open += __popc(und[j]);
         if (A.held && A.lmk && n_open > 0) {
-            if (lane == 0) q0 = atomicAdd(&A.stt->n_scan, (unsigned)n_open);
+            if (lane == 0) q0 = scan_place(atomicAdd(&A.stt->n_scan, (unsigned long long)n_open), A.scan_cap);
             q0 = __shfl_sync(FULL, q0, 0);
-            defer = q0 < A.scan_cap && A.scan_cap - q0 >= (unsigned)n_open;
+            defer = A.scan_cap - q0 >= (unsigned)n_open;
             if (!defer)
                 for (unsigned int i = q0 + lane; i < A.scan_cap && i - q0 < (unsigned)n_open; i += 32)
                     A.scans[i].held = -1;
@@ -1943,7 +1943,7 @@ __global__ void __launch_bounds__(kScanThreads) k_prove_deferred(const LevelArgs
     const unsigned FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
     if (A.stt->arena_overflow) return;  // the level runs again with a larger arena
-    const int count = (int)min(A.stt->n_scan, A.scan_cap);
+    const int count = (int)scan_place(A.stt->n_scan, A.scan_cap);
     const int warps = (int)(gridDim.x * (kScanThreads / 32));
     for (int item = (int)(blockIdx.x * (kScanThreads / 32) + (threadIdx.x >> 5)); item < count; item += warps) {
         const DeferredScan q = A.scans[item];

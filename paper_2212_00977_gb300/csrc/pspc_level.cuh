@@ -85,7 +85,8 @@ struct LevelStatus {
     int n_held;                  // vertices whose segment waits for deferred scans
     int work_scan;
     unsigned int n_scan_open;    // of them, left after the neighbours' proof
-    unsigned int n_scan;         // deferred scans asked for (those past the queue's size run in place)
+    unsigned long long n_scan;   // deferred scans asked for (those past the queue's size run in place): 64 bits,
+                                 // as a level can ask for more than 2^32
     unsigned long long dropped;  // entries that deferred scans took out of their segments
     int max_deg;     // largest degree of the graph (level 2 only)
     int work_dense;
@@ -130,6 +131,11 @@ struct DeferredScan {
     int32_t held;  // which HeldSegment (-1: none)
     int32_t pos;   // which of its entries
 };
+// First place in a queue of `cap` for scans that come after `before` others
+// (cap: it is full).
+__host__ __device__ inline unsigned int scan_place(unsigned long long before, unsigned int cap) {
+    return before < cap ? (unsigned int)before : cap;
+}
 
 // Rows of a distance ball (pspc_ball.cu): row u starts at word off[u] (n + 1
 // values; batches), or at u * words. A multiple of 4 words each; bit r is the
