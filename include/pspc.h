@@ -403,6 +403,12 @@ int pspc_landmarks(const pspc_index* ix, int32_t* k, uint16_t* dist, int32_t* ve
  */
 int pspc_inject_alloc_failure(int64_t after, int32_t status);
 
+/* pspc_inject_alloc_failures -- the same for `count` failing allocations
+ * only, after which allocations succeed again (count < 0: every later one
+ * fails). A build whose failed allocation was for memory that only makes it
+ * faster, or that gives such memory back, goes on. */
+int pspc_inject_alloc_failures(int64_t after, int64_t count, int32_t status);
+
 /* pspc_free -- release an index and all its device memory; NULL is a no-op. */
 void pspc_free(pspc_index* ix);
 

@@ -93,6 +93,7 @@ _SIGS = {
     "pspc_query_noalloc": (ctypes.c_int, [_P, _P, ctypes.c_int64, _P, _P, _P, _P]),
     "pspc_landmarks": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32), _P, _P]),
     "pspc_inject_alloc_failure": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int32]),
+    "pspc_inject_alloc_failures": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int64, ctypes.c_int32]),
     "pspc_free": (None, [_P]),
     "pspc_strerror": (ctypes.c_char_p, [ctypes.c_int]),
 }
@@ -117,14 +118,14 @@ def load(path: str | None = None) -> ctypes.CDLL:
         return lib
 
 
-def inject_alloc_failure(after: int, status: int = PSPC_E_NOMEM) -> None:
-    """pspc_inject_alloc_failure: the library's next ``after`` device
-    allocations succeed and later ones fail with ``status`` (PSPC_E_NOMEM
-    or PSPC_E_CUDA); ``after`` < 0 removes the limit. For tests of the
-    error paths."""
-    rc = load().pspc_inject_alloc_failure(int(after), int(status))
+def inject_alloc_failure(after: int, status: int = PSPC_E_NOMEM, count: int = -1) -> None:
+    """pspc_inject_alloc_failures: the library's next ``after`` device
+    allocations succeed and the ``count`` ones after them (-1: all later
+    ones) fail with ``status`` (PSPC_E_NOMEM or PSPC_E_CUDA); ``after`` < 0
+    removes the limit. For tests of the error paths."""
+    rc = load().pspc_inject_alloc_failures(int(after), int(count), int(status))
     if rc != PSPC_OK:
-        raise PSPCError(rc, "pspc_inject_alloc_failure")
+        raise PSPCError(rc, "pspc_inject_alloc_failures")
 
 
 def strerror(code: int) -> str:

@@ -679,6 +679,10 @@ struct Builder {
     double ball_step_bytes = 0.0;    // read and written by one step
     bool ball_level = false;         // the current level has its ball
     double dup_ratio = 1.0;          // candidates per pulled entry at the last level without one
+    // The balls, the queue of scans and the level kernels' slabs only make a
+    // build faster, or are made anew where a level asks for them: they are
+    // given back when there is no room for what the index needs.
+    bool spare = true;               // balls and the queue may be allocated
     HeldSegment* held = nullptr;     // deferred scans: one segment per vertex at most, and the queue
     DeferredScan* scans = nullptr;   // (and behind it the scans left after the proof)
     unsigned int scan_cap = 0;
@@ -719,17 +723,10 @@ struct Builder {
         dfree(raw_u, st);
         dfree(lab_size, st);
         dfree(items, st);
-        dfree(ball_off, st);
-        dfree(ball[0], st);
-        dfree(ball[1], st);
-        dfree(ball_slices, st);
-        dfree(ball_count, st);
-        dfree(held, st);
-        dfree(scans, st);
+        give_back();
         dfree(glist, st);
         dfree(two_stt, st);
         dfree(err, st);
-        dfree(gscratch, st);
         if (ek0) cudaEventDestroy(ek0);
         if (ek1) cudaEventDestroy(ek1);
         dfree(out.rank, st);
@@ -740,6 +737,42 @@ struct Builder {
         dfree(out.cnt, st);
         dfree(out.lmk, st);
         cudaStreamSynchronize(st);
+    }
+
+    void drop_balls() {
+        dfree(ball_off, st);
+        dfree(ball[0], st);
+        dfree(ball[1], st);
+        dfree(ball_slices, st);
+        dfree(ball_count, st);
+        ball_dist = 0;
+        ball_level = false;
+    }
+
+    void drop_queue() {
+        dfree(held, st);
+        dfree(scans, st);
+    }
+
+    // Whether there was anything to give back.
+    bool give_back() {
+        const bool any = ball[0] || held || gscratch;
+        drop_balls();
+        drop_queue();
+        dfree(gscratch, st);
+        gscratch_bytes = 0;
+        return any;
+    }
+
+    // Memory that the build cannot do without.
+    template <typename T>
+    cudaError_t alloc_needed(T** p, size_t count) {
+        cudaError_t e = dalloc(p, count, st);
+        if (e != cudaErrorMemoryAllocation || !give_back()) return e;
+        cudaGetLastError();
+        spare = false;
+        cudaStreamSynchronize(st);  // what was given back is free now
+        return dalloc(p, count, st);
     }
 
     // The status as of now; ends the level's time (ev_level) here, so that no
@@ -982,8 +1015,8 @@ struct Builder {
         unsigned long long cap = std::max<unsigned long long>(arena_cap * 2, need + need / 4);
         uint32_t* h2 = nullptr;
         uint64_t* c2 = nullptr;
-        PSPC_TRY_CUDA(dalloc(&h2, cap, st));
-        cudaError_t e = dalloc(&c2, cap, st);
+        PSPC_TRY_CUDA(alloc_needed(&h2, cap));
+        cudaError_t e = alloc_needed(&c2, cap);
         if (e != cudaSuccess) {
             dfree(h2, st);
             return cuda_status(e);
@@ -1006,7 +1039,7 @@ struct Builder {
         // storage limit is run to learn whether it is empty)
         int cap = std::max(need, std::min(seg_levels_cap ? seg_levels_cap * 2 : 16, kMaxDist + 2));
         uint64_t* s2 = nullptr;
-        PSPC_TRY_CUDA(dalloc(&s2, (size_t)cap * n, st));
+        PSPC_TRY_CUDA(alloc_needed(&s2, (size_t)cap * n));
         if (seg)
             PSPC_TRY_CUDA(cudaMemcpyAsync(s2, seg, (size_t)seg_levels_cap * n * 8, cudaMemcpyDeviceToDevice, st));
         dfree(seg, st);
@@ -1015,13 +1048,22 @@ struct Builder {
         return PSPC_OK;
     }
 
-    int ensure_gscratch(size_t bytes) {
+    // keep_spare: NOMEM where it would take the balls or the queue.
+    int ensure_gscratch(size_t bytes, bool keep_spare = false) {
         if (bytes <= gscratch_bytes) return PSPC_OK;
         dfree(gscratch, st);
         gscratch_bytes = 0;
-        PSPC_TRY_CUDA(dalloc(&gscratch, bytes, st));
+        PSPC_TRY_CUDA(keep_spare ? dalloc(&gscratch, bytes, st) : alloc_needed(&gscratch, bytes));
         gscratch_bytes = bytes;
         return PSPC_OK;
+    }
+
+    // For a launch with A, whose balls and queue may be gone afterwards.
+    int ensure_gscratch(size_t bytes, LevelArgs& A) {
+        const int rc = ensure_gscratch(bytes);
+        if (!ball_level) A.ball = nullptr;
+        if (!held) A.held = nullptr;
+        return rc;
     }
 
     // Launches the on-chip level kernel over the bucketed vertices, then the
@@ -1063,15 +1105,14 @@ struct Builder {
                                             : d >= kDeferShallow && hstt->raw_total >= kDeferPulled &&
                                                   hstt->n_active >= kDeferActive;
         if (defer && A.lmk && !A.ball) {
-            if (!held) {
+            if (!held && spare) {
                 scan_cap = (unsigned)std::min<int64_t>(std::max<int64_t>(4 * n, 1 << 16), 1 << 26);
                 cudaError_t e = dalloc(&held, n, st);
                 if (e == cudaSuccess) e = dalloc(&scans, 2 * (size_t)scan_cap, st);
-                if (e != cudaSuccess) {  // no room for them: the scans run in place
-                    cudaGetLastError();
-                    dfree(held, st);
-                    held = nullptr;
-                    scans = nullptr;
+                if (e != cudaSuccess) {
+                    drop_queue();
+                    if (cuda_status(e) != PSPC_E_NOMEM) return cuda_status(e);
+                    spare = false;  // no room for them: the scans run in place
                 }
             }
             A.held = held;
@@ -1111,7 +1152,13 @@ struct Builder {
                 dense_grid = std::min(n_dense, sms * (o.granular ? std::max(1, plan.dense_occupancy / 2) : plan.dense_occupancy));
                 dense_grid = (int)std::min<size_t>(dense_grid, std::max<size_t>(1, ((size_t)4 << 30) / slab));
                 if (o.max_ctas > 0) dense_grid = std::min(dense_grid, o.max_ctas);
-                const int rc = ensure_gscratch(slab * dense_grid);
+                // no room: fewer CTAs, and at last without balls and queue
+                int rc = ensure_gscratch(slab * dense_grid, true);
+                while (rc == PSPC_E_NOMEM && dense_grid > 1) {
+                    dense_grid = (dense_grid + 1) / 2;
+                    rc = ensure_gscratch(slab * dense_grid, true);
+                }
+                if (rc == PSPC_E_NOMEM) rc = ensure_gscratch(slab, A);
                 if (rc) return rc;
             }
             cudaEventRecord(ek0, st);
@@ -1204,7 +1251,7 @@ struct Builder {
                 // granular builds leave every SM half free for concurrent work
                 grid = std::min(grid, o.granular ? sms : sms * 2);
                 if (o.max_ctas > 0) grid = std::min(grid, o.max_ctas);
-                rc = ensure_gscratch(stride * grid);
+                rc = ensure_gscratch(stride * grid, A);
                 if (rc) return rc;
                 A.items = pass == 0 ? glist : glist + n;
                 A.n_items = count;
@@ -1335,13 +1382,24 @@ struct Builder {
     // and save 200 a level, so deep graphs keep the filter.
     int use_ball(int d, long long raw) {
         ball_level = false;
-        if (d < 3 || ball_words * 4 > kBallBytes) return PSPC_OK;
+        if (d < 3 || ball_words * 4 > kBallBytes || !spare) return PSPC_OK;
         const int steps = d - 1 - std::max(ball_dist, 1);
         const double cost = (steps + (ball_dist == 0)) * kBallStepSeconds + steps * ball_step_bytes / kBallBytesPerSecond +
                             (ball_dist == 0 ? ball_words * 4.0 / kBallBytesPerSecond : 0.0);
         if (cost >= (double)raw * dup_ratio * (d == 3 ? kRule2Level3 : kRule2Deeper)) return PSPC_OK;
         if (ball_dist == 0) {
-            if (!graph_n.empty()) {
+            cudaError_t e = graph_n.empty() ? cudaSuccess : dalloc(&ball_off, n + 1, st);
+            if (e == cudaSuccess) e = dalloc(&ball[0], ball_words, st);
+            if (e == cudaSuccess) e = dalloc(&ball[1], ball_words, st);
+            if (e == cudaSuccess) e = dalloc(&ball_slices, arcs / 128 + 1, st);
+            if (e == cudaSuccess) e = dalloc(&ball_count, 1, st);
+            if (e != cudaSuccess) {
+                drop_balls();
+                if (cuda_status(e) != PSPC_E_NOMEM) return cuda_status(e);
+                spare = false;  // no room for them: rule 2 as it is without
+                return PSPC_OK;
+            }
+            if (ball_off) {
                 std::vector<int64_t> off;
                 off.reserve((size_t)n + 1);
                 int64_t at = 0;
@@ -1350,14 +1408,9 @@ struct Builder {
                     for (int64_t v = 0; v < m; ++v, at += w) off.push_back(at);
                 }
                 off.push_back(at);
-                PSPC_TRY_CUDA(dalloc(&ball_off, n + 1, st));
                 PSPC_TRY_CUDA(cudaMemcpyAsync(ball_off, off.data(), (n + 1) * 8, cudaMemcpyHostToDevice, st));
                 PSPC_TRY_CUDA(cudaStreamSynchronize(st));  // off is a host buffer of this scope
             }
-            PSPC_TRY_CUDA(dalloc(&ball[0], ball_words, st));
-            PSPC_TRY_CUDA(dalloc(&ball[1], ball_words, st));
-            PSPC_TRY_CUDA(dalloc(&ball_slices, arcs / 128 + 1, st));
-            PSPC_TRY_CUDA(dalloc(&ball_count, 1, st));
             PSPC_TRY_CUDA(launch_ball_init(n, arcs, rp_r, arc_src, col_r, comp_base, {ball_off, ball_row_words}, ball_words,
                                            ball[0], ball_slices, ball_count, st));
             PSPC_TRY_CUDA(cudaMemcpyAsync(&n_ball_slices, ball_count, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1391,8 +1444,8 @@ struct Builder {
             push_hub = nullptr;
             push_cnt = nullptr;
             push_cap = 0;
-            PSPC_TRY_CUDA(dalloc(&push_hub, total + total / 4 + 1, st));
-            PSPC_TRY_CUDA(dalloc(&push_cnt, total + total / 4 + 1, st));
+            PSPC_TRY_CUDA(alloc_needed(&push_hub, total + total / 4 + 1));
+            PSPC_TRY_CUDA(alloc_needed(&push_cnt, total + total / 4 + 1));
             push_cap = total + total / 4 + 1;
         }
         PSPC_TRY_CUDA(launch_push_scatter(arcs, col_r, seg + (int64_t)(d - 1) * n, hub_arena, cnt_arena, cnt_arc,
@@ -1592,6 +1645,7 @@ struct Builder {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         if (rc) return rc;
+        give_back();  // the index arrays come next
         out.levels = levels;
         return PSPC_OK;
     }

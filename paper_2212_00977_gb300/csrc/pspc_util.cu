@@ -31,15 +31,21 @@ static std::mutex g_pool_mu;
 static cudaMemPool_t g_pools[64];
 static bool g_pool_ok[64];
 
-// Allocation-failure injection (pspc_inject_alloc_failure): the number of
-// library device allocations still allowed to succeed, or -1 (no limit).
+// Allocation-failure injection (pspc_inject_alloc_failure, _failures): the
+// number of library device allocations still allowed to succeed, or -1 (no
+// limit), and of those that then fail, or -1 (all).
 static std::atomic<int64_t> g_alloc_budget{-1};
+static std::atomic<int64_t> g_alloc_failures{-1};
 static std::atomic<int> g_alloc_error{(int)cudaErrorMemoryAllocation};  // what an injected failure returns
 
 static bool alloc_allowed() {
     int64_t b = g_alloc_budget.load(std::memory_order_relaxed);
     while (b >= 0) {
-        if (b == 0) return false;
+        if (b == 0) {
+            int64_t f = g_alloc_failures.load(std::memory_order_relaxed);
+            while (f > 0 && !g_alloc_failures.compare_exchange_weak(f, f - 1, std::memory_order_relaxed)) {}
+            return f == 0;
+        }
         if (g_alloc_budget.compare_exchange_weak(b, b - 1, std::memory_order_relaxed)) return true;
     }
     return true;
@@ -178,9 +184,14 @@ int exclusive_scan_i64(int64_t* a, int64_t n, cudaStream_t st, int64_t* launches
 using namespace pspc;
 
 extern "C" int pspc_inject_alloc_failure(int64_t after, int32_t status) {
+    return pspc_inject_alloc_failures(after, -1, status);
+}
+
+extern "C" int pspc_inject_alloc_failures(int64_t after, int64_t count, int32_t status) {
     if (status != PSPC_E_NOMEM && status != PSPC_E_CUDA) return PSPC_E_INVAL;
     g_alloc_error.store(status == PSPC_E_NOMEM ? (int)cudaErrorMemoryAllocation : (int)cudaErrorInvalidValue,
                         std::memory_order_relaxed);
+    g_alloc_failures.store(count < 0 ? -1 : count, std::memory_order_relaxed);
     g_alloc_budget.store(after < 0 ? -1 : after, std::memory_order_relaxed);
     return PSPC_OK;
 }

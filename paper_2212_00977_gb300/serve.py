@@ -41,7 +41,9 @@ def estimate_index_bytes(n: int, arcs: int) -> int:
     """Conservative device footprint of a build: label entries are estimated
     as n * (10 + 4 * avg_degree * log2(n)) (above what R-MAT and
     Barabasi-Albert graphs produce), at 14 bytes in the index plus 12 in the
-    build arena, plus 24 bytes per arc of working arrays."""
+    build arena, plus 24 bytes per arc of working arrays. Not in it: distance
+    balls, level-kernel slabs (up to 4 GiB each) and the queue of scans,
+    which a build does without, or gives back, where there is no room."""
     avg_deg = arcs / max(n, 1)
     entries = n * (10 + 4 * avg_deg * math.log2(max(n, 2)))
     return int(entries * 26 + arcs * 24 + n * 64)
