@@ -1772,10 +1772,8 @@ struct Builder {
             out.launches += 1;
             PSPC_TRY_CUDA(cudaGetLastError());
         }
-        unsigned long long hovf[2] = {0, 0};
-        PSPC_TRY_CUDA(cudaMemcpyAsync(hovf, n_ovf, 16, cudaMemcpyDeviceToHost, st));
+        PSPC_TRY_CUDA(cudaMemcpyAsync(&out.overflow_entries, n_ovf, 8, cudaMemcpyDeviceToHost, st));
         PSPC_TRY_CUDA(cudaStreamSynchronize(st));
-        out.overflow_entries = (int64_t)hovf[0];
         dfree(big, st);
         dfree(ctr, st);
         dfree(d_lvl, st);

@@ -404,34 +404,31 @@ static int export_on_host(const Index& ix, int64_t* off, int32_t* hub, uint16_t*
 }
 
 // The same in chunks gathered on the device, each copied to its place in the
-// caller's arrays. *no_room: the scratch was not to be had and nothing that
-// matters was written.
+// caller's arrays. *no_room: the device has no memory for the scratch, and
+// nothing that matters was written.
 static int export_gathered(const Index& ix, int64_t* off, int32_t* hub, uint16_t* dist, uint64_t* cnt, uint8_t* ovf,
                            bool* no_room) {
     const cudaStream_t st = 0;
     const int64_t n = ix.n;
     int64_t* d_pos = nullptr;
     uint64_t* d_cnt = nullptr;
-    *no_room = dev_alloc((void**)&d_pos, (n + 1) * 8, st) != cudaSuccess;
-    if (*no_room) {
-        cudaGetLastError();
-        return PSPC_OK;
-    }
-    // every vertex is in range: no error is ever flagged
-    k_vert_sizes<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, nullptr, n, ix.rank, ix.off, d_pos, nullptr);
-    cudaError_t e = cudaGetLastError();
-    int rc = e == cudaSuccess ? exclusive_scan_i64(d_pos, n, st) : cuda_status(e);
-    if (rc != PSPC_OK) *no_room = true;
+    int rc = cuda_status(dev_alloc((void**)&d_pos, (n + 1) * 8, st));
     if (rc == PSPC_OK) {
-        e = cudaMemcpyAsync(off, d_pos, (n + 1) * 8, cudaMemcpyDeviceToHost, st);
+        // every vertex is in range: no error is ever flagged
+        k_vert_sizes<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, nullptr, n, ix.rank, ix.off, d_pos, nullptr);
+        rc = cuda_status(cudaGetLastError());
+    }
+    if (rc == PSPC_OK) rc = exclusive_scan_i64(d_pos, n, st);
+    if (rc == PSPC_OK) {
+        cudaError_t e = cudaMemcpyAsync(off, d_pos, (n + 1) * 8, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         int64_t cap = std::min<int64_t>(ix.entries, kExportChunk);
         for (int64_t v = 0; e == cudaSuccess && v < n; ++v) cap = std::max(cap, off[v + 1] - off[v]);
-        if (e == cudaSuccess && cap > 0 && dev_alloc((void**)&d_cnt, cap * 15, st) != cudaSuccess) *no_room = true;
+        if (e == cudaSuccess && cap > 0) e = dev_alloc((void**)&d_cnt, cap * 15, st);
         int32_t* d_hub = (int32_t*)(d_cnt + cap);
         uint16_t* d_dist = (uint16_t*)(d_hub + cap);
         uint8_t* d_ovf = (uint8_t*)(d_dist + cap);
-        for (int64_t v = 0; e == cudaSuccess && !*no_room && v < n;) {
+        for (int64_t v = 0; e == cudaSuccess && v < n;) {
             const int64_t p = off[v];
             const int64_t to = std::upper_bound(off + v + 1, off + n + 1, p + cap) - off - 1;  // > v: cap holds any label
             const int64_t E = off[to] - p;
@@ -448,14 +445,11 @@ static int export_gathered(const Index& ix, int64_t* off, int32_t* hub, uint16_t
             }
             v = to;
         }
-        if (e != cudaSuccess) rc = cuda_status(e);
+        rc = cuda_status(e);
     }
     dev_free(d_pos, st);
     dev_free(d_cnt, st);
-    if (*no_room) {
-        cudaGetLastError();
-        return PSPC_OK;
-    }
+    *no_room = rc == PSPC_E_NOMEM;
     return rc;
 }
 

@@ -51,3 +51,22 @@ def test_device_and_host_forms_agree(pspc, name):  # noqa: F811
                 assert a.dtype == b.dtype and np.array_equal(a, b)
     finally:
         ix.free()
+
+
+@pytest.mark.parametrize("name", ["isolated", "grid100"])
+def test_other_errors_are_reported(pspc, name):  # noqa: F811
+    """The host form is for a device without room, not for a CUDA error."""
+    g, rank = GRAPHS[name]()
+    ix = pspc.Index.from_graph(g, rank)
+    try:
+        for failing in range(3 if name == "grid100" else 2):  # the scan allocates beyond 4,096 vertices
+            pspc.inject_alloc_failure(failing, pspc.PSPC_E_CUDA)
+            try:
+                with pytest.raises(pspc.PSPCError) as e:
+                    ix.export()
+            finally:
+                pspc.inject_alloc_failure(-1)
+            assert e.value.code == pspc.PSPC_E_CUDA
+        assert len(ix.export()[1]) == ix.stats()["entries"]
+    finally:
+        ix.free()
