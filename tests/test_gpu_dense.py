@@ -25,17 +25,40 @@ def pspc():
     return lib
 
 
-@pytest.mark.parametrize("scale,ef,order,kw", [
+WINDOWS = [
     (15, 8, "degree", {}),                    # three windows of ids
-    (14, 16, "random", {}),                   # hubs anywhere: long rows over two windows, no table of window starts
+    (14, 16, "random", {}),                   # hubs anywhere: long rows over several windows, no table of window starts
     (14, 16, "degree", {"granular": True}),   # only the heaviest vertices
     (14, 8, "degree", {"landmarks": -1}),     # every candidate goes to the label scans
     (13, 16, "degree", {"max_ctas": 3}),      # a few CTAs take every vertex
-])
+]
+
+
+@pytest.mark.parametrize("scale,ef,order,kw", WINDOWS)
 def test_windows_and_rows(pspc, scale, ef, order, kw):
+    """With distance balls, whose rows stand for the member bitmaps and for
+    rule 2, at level 3."""
     g = P.rmat(scale, ef, *P.RMAT_ABCD, seed=5)
     rank = P.degree_rank(g, "id") if order == "degree" else G.random_rank(g.n, 4)
     ix = gpu_index(pspc, g, rank, **kw)
+    level = ix.level_stats()[2]
+    assert level["unique_candidates"] == level["entries"]
+    _check_whole_index(g, rank, *ix.export())
+    ix.free()
+
+
+@pytest.mark.parametrize("scale,ef,order,kw", WINDOWS)
+def test_windows_and_rows_without_balls(pspc, scale, ef, order, kw):
+    """The same graphs among isolated vertices, too many for balls: member
+    bitmaps, the marking walk of level 3 (in two rounds of ids where the
+    graph's are spread over all of them), the filter and the scans."""
+    g = P.rmat(scale, ef, *P.RMAT_ABCD, seed=5)
+    n = 170_000 if order == "random" else 131_100
+    g = P.csr_from_edges(n, g.edges(), "among isolated")
+    rank = P.degree_rank(g, "id") if order == "degree" else G.random_rank(g.n, 4)
+    ix = gpu_index(pspc, g, rank, **kw)
+    for level in ix.level_stats()[2:4]:
+        assert level["unique_candidates"] > level["entries"] and level["raw_candidates"] > 1 << 19
     _check_whole_index(g, rank, *ix.export())
     ix.free()
 
