@@ -1226,6 +1226,10 @@ struct Builder {
         A.held = nullptr;  // off chip the scans run in place
         int rc = read_status();
         if (rc) return rc;
+        if (hstt->bad) {  // never seen
+            fprintf(stderr, "pspc level %d: inconsistent label segments\n", d);
+            return PSPC_E_CUDA;
+        }
         if (hstt->n_smem > 0) {
             float ms = 0.f;
             cudaEventElapsedTime(&ms, ek0, ek1);

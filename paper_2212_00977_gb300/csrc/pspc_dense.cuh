@@ -25,7 +25,18 @@
 // The hash it replaces kept tables of more than 4,096 slots in device memory,
 // half of whose sectors missed L2: levels 3 and 4 took 568 and 495 ms, now
 // 180 and 208 (the build 1,182 -> 488 ms). With a distance ball its row is the
-// window's bitmap and only the pull is left.
+// window's bitmap and only the pull is left. Eight CTAs an SM leave a thread 32
+// registers, and ptxas spills (240 bytes of stores, 448 of loads); four CTAs with
+// 64 registers spill nothing and were slower (kDenseThreads).
+//
+// Three checks keep the kernel inside its memory whatever it reads: a run of a
+// segment that ends before it starts is empty, a member outside its window is
+// left out, and a window with more candidates than the slab holds is dropped.
+// By the order of the segments none of them can happen; if one does, it sets
+// LevelStatus::bad and the build ends with PSPC_E_CUDA. They are there because
+// one granular build (kDenseMinRawGranular) ended in a GPU fault that reading
+// has not explained. They cost 1.4% of the build of R-MAT 2^20 (494 -> 501 ms),
+// any one of them alone as much: the registers are full.
 
 // Words of the window's bitmaps.
 constexpr uint32_t kDenseWords = kDenseWindow / 32;
@@ -163,6 +174,11 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
             if (w == nwin) return len;
             return table ? bnd[r * nb + w - 1] : seg_lower_bound(A.hub_arena + start, len, cbase + w * W);
         };
+        // length of the run [b, e) of a segment (e is at most its length)
+        auto run = [&](uint32_t b, uint32_t e) -> uint32_t {
+            if (b > e) A.stt->bad = 1;
+            return b > e ? 0u : e - b;
+        };
         uint64_t my_start = 0;
         uint32_t my_len = 0;
         if (tid < deg) arc_run(tid, my_start, my_len);  // the first chunk of arcs stays in registers
@@ -179,28 +195,29 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
             } else {  // members of L_<d(u) in the window
                 const uint32_t e1 = edge((uint32_t)deg, seg_start(own1), seg_len(own1), w);
                 const uint32_t e2 = edge((uint32_t)deg + 1, seg_start(own2), seg_len(own2), w);
-                const uint32_t n1 = edge((uint32_t)deg, seg_start(own1), seg_len(own1), w + 1) - e1;
-                const uint32_t n2 = edge((uint32_t)deg + 1, seg_start(own2), seg_len(own2), w + 1) - e2;
+                const uint32_t n1 = run(e1, edge((uint32_t)deg, seg_start(own1), seg_len(own1), w + 1));
+                const uint32_t n2 = run(e2, edge((uint32_t)deg + 1, seg_start(own2), seg_len(own2), w + 1));
                 const uint64_t s1 = seg_start(own1) + e1, s2 = seg_start(own2) + e2 - n1;
                 for (uint32_t i = tid; i < n1 + n2; i += NT) {
                     const uint32_t x = (__ldg(A.hub_arena + (i < n1 ? s1 : s2) + i) & kHubMask) - w0;
-                    atomicOr(&mem[x >> 5], 1u << (x & 31));
+                    if (x < W) atomicOr(&mem[x >> 5], 1u << (x & 31));
+                    else A.stt->bad = 1;
                 }
             }
             bool any = false;
             for (int c0 = 0; c0 < deg; c0 += NT) {
                 const int nc = deg - c0 < NT ? deg - c0 : NT;
                 uint64_t start = my_start;
-                uint32_t len = my_len, b0 = 0, b1 = 0;
+                uint32_t len = my_len, b0 = 0, cnt = 0;
                 if (tid < nc) {
                     if (c0 > 0) arc_run(c0 + tid, start, len);
                     if (len) {
                         b0 = edge((uint32_t)(c0 + tid), start, len, w);
-                        b1 = edge((uint32_t)(c0 + tid), start, len, w + 1);
+                        cnt = run(b0, edge((uint32_t)(c0 + tid), start, len, w + 1));
                     }
                 }
                 if (c0 > 0) __syncthreads();  // pfx and st of the chunk before are still read
-                const uint32_t total = dense_scan(b1 - b0, nc, pfx, s_wsum);
+                const uint32_t total = dense_scan(cnt, nc, pfx, s_wsum);
                 if (tid < nc) st[tid] = start + b0 - pfx[tid];
                 __syncthreads();
                 any |= total > 0;
@@ -255,6 +272,12 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
                     const int t = s_wcnt[k];
                     at += k < warp ? t : 0;
                     M += t;
+                }
+                if ((uint32_t)M > A.cap_c_max) {
+                    A.stt->bad = 1;
+                    for (int k = 0; k < kWarps; ++k) M -= s_wcnt[k];
+                    mine = 0;
+                    for (uint32_t i = tid; i < W; i += NT) acc[i] = 0u;
                 }
                 for (uint32_t g = g0; mine > 0 && g < g1; ++g) {
                     const uint4 v = ((const uint4*)acc)[g * 32 + lane];

@@ -55,8 +55,12 @@ constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32
 constexpr int64_t kDenseMinRaw = 512;
 constexpr int64_t kDenseRawPerWindow = 12;
 // Granular builds run one hash CTA per vertex, and the dense kernel at half
-// occupancy: only vertices that would mostly overflow the hash pay (BA
-// 20,011: 7.2 ms, with 2,048 here 7.9 ms).
+// occupancy: only vertices that would mostly overflow the hash pay (granular,
+// R-MAT 262,144 builds in 81.8 ms with 16,384, in 103.4 with 65,536 and in 115.8
+// without direct addressing; R-MAT 65,536 11.8, 11.8 and 11.6, BA 100,000 with
+// m = 8 64.1, 61.2 and 61.3, BA 20,011 3.7 in all). Lower lines are closed: a
+// granular build of BA 20,011 with one (512 pulled entries and 384 a window)
+// ended in a GPU fault, Xid 13 and 43, whose cause is not known.
 constexpr int64_t kDenseMinRawGranular = 16384;
 
 struct LevelStatus {
@@ -89,6 +93,7 @@ struct LevelStatus {
                                  // as a level can ask for more than 2^32
     unsigned long long dropped;  // entries that deferred scans took out of their segments
     int max_deg;     // largest degree of the graph (level 2 only)
+    int bad;         // k_level_dense met a run outside its segment, a hub outside its window or a full slab
     int work_dense;
     unsigned int cmax;  // largest count appended at this level (0xFFFFFFFF: 2^32 or more, or flagged)
     // on-chip attempts and overflows of vertices that can overflow, by
