@@ -16,10 +16,11 @@
 // overflow flag) times u's degree is below 2^32. The other vertices keep the
 // hash kernels with 64-bit sums, carries and flags.
 //
-// What bounds it: latency. On R-MAT 262,144, level 3, with half the warps it
-// has now, 40% of the issue slots were used, of 20 cycles per issue 8 waited
-// for reads (L2 hits half of the time), 4 at barriers; DRAM was at 12%, L2 at
-// 10%. By phases, on R-MAT 2^20, level 3 (3.0e10 pulled entries): half pull, a
+// What bounds it: latency and instructions. On R-MAT of 140,000 vertices, level
+// 3, all 64 warps of an SM are there and 65% of the issue slots are used; of 24
+// cycles between a warp's instructions 9 wait for reads (L2 hits 73% of them)
+// and 6 at barriers; DRAM is at 8%, L2 at 26%, L1 at 50%. With four CTAs, half
+// the warps, it was 41% on R-MAT 262,144. By phases, before that, on R-MAT 2^20, level 3 (3.0e10 pulled entries): half pull, a
 // fifth the marking walk, a tenth each the member bitmaps and the scans of
 // run lengths; at level 4 the landmark filter and the label scans take 57%.
 // The hash it replaces kept tables of more than 4,096 slots in device memory,

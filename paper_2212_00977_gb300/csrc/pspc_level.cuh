@@ -17,7 +17,9 @@ constexpr uint32_t kOffStartCap = 16384;    // first off-chip table size
 constexpr uint32_t kOffSlabCap = 1u << 17;  // off-chip slab of the first pass, in candidate slots
 constexpr int kMicroThreads = 256;    // the warp-per-vertex level kernel: 8 vertices per CTA
 constexpr int kMicroBucket = 7;       // micro: fewer than 2^7 pulled entries (four to a lane); at levels 2 and 3,
-                                      // where nothing is filtered out first, 2^6 (BA 20,011: 6.7 ms, else 6.9)
+                                      // where nothing is filtered out first, 2^6. Since levels use balls either line
+                                      // does there: R-MAT 262,144 builds in 49.1 ms, with 2^7 in 49.3, BA 20,011 in
+                                      // 2.91 both ways, the batch of 96 BA graphs in 80.0 and 78.1
 constexpr int kTinyBucket = 6;        // of those, fewer than 2^6: two to a lane, and fewer registers
 constexpr int kLightBucket = 9;       // light: fewer than 2^9 pulled entries, so at most 2 * 511 < kLightCap
                                       // slots are asked for, and the table never overflows
@@ -38,7 +40,7 @@ constexpr int kLmkDeepLevel = 16;  // from this level on, the filter tests every
 // with 4,608-id windows fill each other's gaps best: R-MAT 2^20 builds in 488
 // ms, with 4 CTAs and 11,264 ids 578, 5 and 8,960 547, 6 and 6,912 505, 7 and
 // 5,760 515, 4 of 512 threads and 10,240 ids 496 (batch of 96 BA graphs 83 ms,
-// 91, 90, 86, 86 and 92).
+// 91, 90, 86, 86 and 92; all before the kernel's checks).
 constexpr int kDenseThreads = 256;
 constexpr int kDenseBlocks = 8;             // resident CTAs per SM (26 KB of shared memory each)
 constexpr uint32_t kDenseWindow = 4608;     // ids per on-chip window, a multiple of 128
@@ -46,12 +48,11 @@ constexpr uint32_t kDenseBounds = 1024;     // cells of the table of window star
 constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (32 MB of slab a CTA)
 constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32 + floor(log2 pulled entries)
 // A vertex with fewer pulled entries has too few to pay for the windows; it
-// is one of the light class then. A batch of 96 BA graphs builds in 92 ms with
-// 512 here, 95 with 256, 97 with 768, 102 with 1,024, 109 with 2,048 (R-MAT
-// 262,144 59.0, 59.7, 59.6, 61.2 and 63.7 ms, BA 20,011 3.12, 3.12, 3.21, 3.32
-// and 3.55; all with windows of 11,264 ids). Per window of its id range it
-// needs 12 (window overhead against a hash in device memory): R-MAT 2^20 488
-// ms with 12, 494 with 20.
+// is one of the light class then. A batch of 96 BA graphs builds in 80.0 ms with
+// 512 here, 81.6 with 256, 87.3 with 768, 91.7 with 1,024, 99.9 with 2,048 (R-MAT
+// 262,144 49.1, 48.5, 50.0, 50.7 and 54.5 ms, BA 20,011 2.91, 2.93, 3.02, 3.13
+// and 3.43). Per window of its id range it needs 12 (window overhead against a
+// hash in device memory): R-MAT 2^20 496 ms with 12 and with 6, 504 with 20.
 constexpr int64_t kDenseMinRaw = 512;
 constexpr int64_t kDenseRawPerWindow = 12;
 // Granular builds run one hash CTA per vertex, and the dense kernel at half
@@ -105,21 +106,26 @@ struct LevelStatus {
     int bucket_fill[kBuckets];
 };
 
-// Deferred label scans. A vertex with undecided
-// candidates appends them with its survivors and asks for their scans; the
+// Deferred label scans. A vertex with undecided candidates appends them with its survivors and asks for their scans; the
 // scans of all vertices then run evenly over the GPU (k_scan_deferred), and
 // the last one of a vertex closes its segment.
 constexpr int kDeferLevel = 16;  // from this level on
 // and with this many active vertices times levels, where the scans are
-// worth two launches a level (grid 61x67 builds in 17.2 ms without them, 17.9
-// with 2^17 here; grid 128x128 54 ms either way, grid 256x256 339 and 336).
+// worth two launches a level. Builds with 2^17, 2^18 and 2^19 here, and without
+// deferral from this level on: grid 61x67 11.9, 11.1, 11.1 and 11.1 ms, 90x90
+// 20.3, 20.4, 20.8 and 20.8, 128x128 37.0, 37.7, 39.5 and 52, 181x181 78.5, 80.4,
+// 85.2 and 179, 256x256 241, 242, 243 and 742.
 constexpr int64_t kDeferWork = 1 << 18;
 // Before it, with this many pulled entries and active vertices: a vertex with
 // a hundred undecided candidates scans for them one after another while the
 // GPU is idle (R-MAT 65,536, level 5: 788,080 pulled, 2.5 ms in place and 0.4
 // deferred). The queue, its allocation and two launches cost some 60 us: of
-// BA 100,000, level 8, 61,290 pulled take 0.18 ms in place and 0.21 deferred,
-// and BA 2,000 builds in 1.04 ms without it, 1.10 with.
+// BA 100,000, level 8, 61,290 pulled take 0.18 ms in place and 0.21 deferred.
+// Builds with 1,024, 2,048 and 4,096 active vertices as the line, and without
+// deferral before kDeferLevel: R-MAT 65,536 8.73, 8.73, 9.17 and 9.63 ms, 6,000
+// 1.23, 1.24, 1.28 and 1.27, BA 40,000 (m = 3) 5.47, 5.47, 5.48 and 5.97, BA 2,000
+// 1.10, 1.04, 1.05 and 1.04; within 2% whatever the line for BA of 3,000, 4,500,
+// 9,000 and 100,000 vertices and R-MAT of 3,000, 12,000 and 24,000.
 constexpr int kDeferShallow = 4;
 constexpr unsigned long long kDeferPulled = 1 << 18;
 constexpr int kDeferActive = 2048;
