@@ -19,7 +19,7 @@
 // What bounds it: latency and instructions. On R-MAT of 140,000 vertices, level
 // 3, all 64 warps of an SM are there and 65% of the issue slots are used; of 24
 // cycles between a warp's instructions 9 wait for reads (L2 hits 73% of them)
-// and 6 at barriers; DRAM is at 8%, L2 at 26%, L1 at 50%. With four CTAs, half
+// and 6 at barriers; DRAM is at 8%, L2 at 25%, L1 at 49%. With four CTAs, half
 // the warps, it was 41% on R-MAT 262,144. By phases, before that, on R-MAT 2^20, level 3 (3.0e10 pulled entries): half pull, a
 // fifth the marking walk, a tenth each the member bitmaps and the scans of
 // run lengths; at level 4 the landmark filter and the label scans take 57%.
@@ -27,17 +27,18 @@
 // half of whose sectors missed L2: levels 3 and 4 took 568 and 495 ms, now
 // 180 and 208 (the build 1,182 -> 488 ms). With a distance ball its row is the
 // window's bitmap and only the pull is left. Eight CTAs an SM leave a thread 32
-// registers, and ptxas spills (240 bytes of stores, 448 of loads); four CTAs with
+// registers, and ptxas spills (220 bytes of stores, 352 of loads); four CTAs with
 // 64 registers spill nothing and were slower (kDenseThreads).
 //
 // Three checks keep the kernel inside its memory whatever it reads: a run of a
 // segment that ends before it starts is empty, a member outside its window is
-// left out, and a window with more candidates than the slab holds is dropped.
+// left out, and a vertex with more candidates than the slab holds is dropped.
 // By the order of the segments none of them can happen; if one does, it sets
 // LevelStatus::bad and the build ends with PSPC_E_CUDA. They are there because
 // one granular build (kDenseMinRawGranular) ended in a GPU fault that reading
-// has not explained. They cost 1.4% of the build of R-MAT 2^20 (494 -> 501 ms),
-// any one of them alone as much: the registers are full.
+// has not explained. They cost nothing (R-MAT 2^20 489 ms with and without) as
+// long as the last one leaves the windows: going on after it, with the counts
+// cleared on the spot, took 497.
 
 // Words of the window's bitmaps.
 constexpr uint32_t kDenseWords = kDenseWindow / 32;
@@ -275,10 +276,11 @@ __global__ void __launch_bounds__(kDenseThreads, kDenseBlocks) k_level_dense(con
                     M += t;
                 }
                 if ((uint32_t)M > A.cap_c_max) {
-                    A.stt->bad = 1;
-                    for (int k = 0; k < kWarps; ++k) M -= s_wcnt[k];
-                    mine = 0;
-                    for (uint32_t i = tid; i < W; i += NT) acc[i] = 0u;
+                    if (tid == 0) A.stt->bad = 1;
+                    M = 0;
+                    dirty = W;
+                    __syncthreads();
+                    break;
                 }
                 for (uint32_t g = g0; mine > 0 && g < g1; ++g) {
                     const uint4 v = ((const uint4*)acc)[g * 32 + lane];

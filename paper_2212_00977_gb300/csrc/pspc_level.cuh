@@ -18,8 +18,8 @@ constexpr uint32_t kOffSlabCap = 1u << 17;  // off-chip slab of the first pass, 
 constexpr int kMicroThreads = 256;    // the warp-per-vertex level kernel: 8 vertices per CTA
 constexpr int kMicroBucket = 7;       // micro: fewer than 2^7 pulled entries (four to a lane); at levels 2 and 3,
                                       // where nothing is filtered out first, 2^6. Since levels use balls either line
-                                      // does there: R-MAT 262,144 builds in 49.1 ms, with 2^7 in 49.3, BA 20,011 in
-                                      // 2.91 both ways, the batch of 96 BA graphs in 80.0 and 78.1
+                                      // does there: R-MAT 262,144 builds in 48.2 ms, with 2^7 in 48.4, BA 20,011 in
+                                      // 2.91 both ways, the batch of 96 BA graphs in 79.6 and 77.9
 constexpr int kTinyBucket = 6;        // of those, fewer than 2^6: two to a lane, and fewer registers
 constexpr int kLightBucket = 9;       // light: fewer than 2^9 pulled entries, so at most 2 * 511 < kLightCap
                                       // slots are asked for, and the table never overflows
@@ -48,17 +48,17 @@ constexpr uint32_t kDenseBounds = 1024;     // cells of the table of window star
 constexpr uint32_t kDenseSlabCap = 1u << 21;  // candidates of one vertex at most (32 MB of slab a CTA)
 constexpr int kDenseBucket = 32;            // dense vertices are bucketed at 32 + floor(log2 pulled entries)
 // A vertex with fewer pulled entries has too few to pay for the windows; it
-// is one of the light class then. A batch of 96 BA graphs builds in 80.0 ms with
-// 512 here, 81.6 with 256, 87.3 with 768, 91.7 with 1,024, 99.9 with 2,048 (R-MAT
-// 262,144 49.1, 48.5, 50.0, 50.7 and 54.5 ms, BA 20,011 2.91, 2.93, 3.02, 3.13
+// is one of the light class then. A batch of 96 BA graphs builds in 79.6 ms with
+// 512 here, 81.3 with 256, 87.2 with 768, 91.5 with 1,024, 99.7 with 2,048 (R-MAT
+// 262,144 48.2, 47.5, 49.1, 49.9 and 53.8 ms, BA 20,011 2.91, 2.93, 3.02, 3.13
 // and 3.43). Per window of its id range it needs 12 (window overhead against a
-// hash in device memory): R-MAT 2^20 496 ms with 12 and with 6, 504 with 20.
+// hash in device memory): R-MAT 2^20 487 ms with 12, 486 with 6, 494 with 20.
 constexpr int64_t kDenseMinRaw = 512;
 constexpr int64_t kDenseRawPerWindow = 12;
 // Granular builds run one hash CTA per vertex, and the dense kernel at half
 // occupancy: only vertices that would mostly overflow the hash pay (granular,
-// R-MAT 262,144 builds in 81.8 ms with 16,384, in 103.4 with 65,536 and in 115.8
-// without direct addressing; R-MAT 65,536 11.8, 11.8 and 11.6, BA 100,000 with
+// R-MAT 262,144 builds in 81.6 ms with 16,384, in 103.2 with 65,536 and in 112.7
+// without direct addressing; R-MAT 65,536 11.8, 11.8 and 11.5, BA 100,000 with
 // m = 8 64.1, 61.2 and 61.3, BA 20,011 3.7 in all). Lower lines are closed: a
 // granular build of BA 20,011 with one (512 pulled entries and 384 a window)
 // ended in a GPU fault, Xid 13 and 43, whose cause is not known.
