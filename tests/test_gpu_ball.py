@@ -1,6 +1,6 @@
 """Levels that prune by distance balls: every entry of the index equals the
-oracle's or the definition's on graphs whose levels use them from level 3, in
-between, or not at all; rows longer than a warp's slice; batches of graphs of
+oracle's or the definition's on graphs whose levels use them from level 3 or
+only in between; rows longer than a warp's slice; batches of graphs of
 very different sizes; balls caught up over several levels."""
 from __future__ import annotations
 
@@ -36,6 +36,32 @@ def test_single_graphs(pspc, make):  # noqa: F811
         ix = gpu_index(pspc, g, rank, **kw)
         _check_whole_index(g, rank, *ix.export())
         ix.free()
+
+
+def _sparse(n, seed):
+    e = np.random.default_rng(seed).integers(0, n, (3 * n // 2, 2))
+    return P.csr_from_edges(n, e[e[:, 0] != e[:, 1]], "sparse")
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_balls_caught_up(pspc, batch):  # noqa: F811
+    """Sparse random graphs, whose candidates are few at first: the first
+    level with a ball brings it four steps or more at once, and the last
+    levels go without."""
+    graphs = [_sparse(n, 3) for n in ((4000, 2500) if batch else (4000,))]
+    ranks = [G.random_rank(g.n, 6) for g in graphs]
+    if batch:
+        ix = pspc.Index.build_batch([(g.n, g.row_ptr, g.col, r) for g, r in zip(graphs, ranks)])
+    else:
+        ix = gpu_index(pspc, graphs[0], ranks[0])
+    by_ball = [l["unique_candidates"] == l["entries"] > 1 << 15 and l["landmark_pruned"] == 0 for l in ix.level_stats()]
+    assert not any(by_ball[2:5]) and any(by_ball[5:8]) and not any(by_ball[-3:])
+    base = 0
+    for g, r in zip(graphs, ranks):
+        off, hub, dist, cnt, ovf = ix.export_vertices(np.arange(base, base + g.n, dtype=np.int32))
+        _check_whole_index(g, r, off, hub - base, dist, cnt, ovf)
+        base += g.n
+    ix.free()
 
 
 def test_batch_of_uneven_graphs(pspc):  # noqa: F811

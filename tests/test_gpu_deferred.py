@@ -11,7 +11,7 @@ import pytest
 import oracle
 import pspc_inputs as P
 from tests import _graphs as G
-from tests.test_gpu_parity import assert_index_equal, gpu_index, pspc  # noqa: F401
+from tests.test_gpu_parity import _check_whole_index, assert_index_equal, gpu_index, pspc  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -29,6 +29,16 @@ def test_deferred_scans(pspc, name, order):  # noqa: F811
         ls = ix.level_stats()
         assert sum(l["entries"] for l in ls) + g.n == len(ref.hub)
         ix.free()
+
+
+@pytest.mark.parametrize("kw", [{}, {"warp_levels": -1}])
+def test_more_scans_than_the_queue_holds(pspc, kw):  # noqa: F811
+    g, rank, _ = P.workload("grid100")
+    ix = gpu_index(pspc, g, rank, landmarks=1, **kw)
+    undecided = [l["unique_candidates"] - l["landmark_pruned"] - l["landmark_proven"] for l in ix.level_stats()]
+    assert max(undecided) > max(4 * g.n, 1 << 16)
+    _check_whole_index(g, rank, *ix.export())
+    ix.free()
 
 
 def test_odd_cycles(pspc):  # noqa: F811
